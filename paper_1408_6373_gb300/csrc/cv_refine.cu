@@ -614,10 +614,11 @@ cudaError_t launch_batch_reset(const BatchItem *items, const CombineArgs *cargs,
     return cudaGetLastError();
 }
 
-// Copy the states of the listed integrals into one contiguous array.
+// Copy the states of the listed integrals (null list: of all of them, in
+// order) into one contiguous array.
 __global__ void k_gather_states(const BatchItem *items, const int *list, DevState *out)
 {
-    const int *src = reinterpret_cast<const int *>(items[list[blockIdx.x]].st);
+    const int *src = reinterpret_cast<const int *>(items[list ? list[blockIdx.x] : (int)blockIdx.x].st);
     int *dst = reinterpret_cast<int *>(out + blockIdx.x);
     for (int i = threadIdx.x; i < (int)(sizeof(DevState) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
 }
