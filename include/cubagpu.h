@@ -499,7 +499,7 @@ void cv_integral_destroy(cv_integral *I);
  * FP32 path only (CV_FP64 / CV_PLAIN are rejected); ndim * nbins must fit
  * the per-warp histograms in shared memory (10 * ndim * nbins * 4 bytes
  * <= 227 KiB, e.g. 32 x 128 or 20 x 256).  An integral's points are cut
- * into tiles by a rule that depends on that integral alone (about 16
+ * into tiles by a rule that depends on that integral alone (at most 32
  * tiles per iteration, 2^11 .. cap points each; CUBAGPU_TILE, points,
  * forces one size), and each tile leaves its sums and histogram as
  * partial rows that the refinement and combination add in tile order (no

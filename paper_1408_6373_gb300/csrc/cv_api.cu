@@ -1548,20 +1548,56 @@ static cudaError_t dispatch_batch_occupancy(int ndim, bool pow2, int stride, int
 }  // namespace cv
 
 // Tile size, in 32-point blocks, of one integral's iteration of n points:
-// about 16 tiles per iteration, a power of two between 64 and cap.  It
-// depends on the integral alone, so a batch or a serving round never
-// changes how an integral's points are grouped and summed.
-// Tile of an iteration of n points: the smallest power of two >= 64
-// blocks that cuts the iteration into at most `split` tiles, capped at
-// `cap` blocks.  A tile is shared evenly by a CTA's eight warps, so the
-// points each thread takes from a tile are tile / 8: split and cap set the
-// points per thread (the autotuner picks both).
-static int tile_blocks_for(long long n, int cap, int split = 16)
+// the smallest power of two >= 64 blocks that cuts the iteration into at
+// most `split` tiles, capped at `cap` blocks.  It depends on the integral
+// alone, so a batch or a serving round never changes how an integral's
+// points are grouped and summed.  A tile is shared evenly by a CTA's eight
+// warps, so the points each thread takes from a tile are tile / 8: split
+// and cap set the points per thread (the autotuner picks both).
+static int tile_blocks_for(long long n, int cap, int split)
 {
     const long long blocks = (n + 31) / 32 + 1;
     long long t = 64;
     while (t < cap && t * split < blocks) t <<= 1;
     return (int)t;
+}
+
+// Defaults of the rule.  A tile costs ~5 us of a CTA besides its points,
+// and a launch's end is as long as its last tiles, so the best size is
+// between: every tile 2^11 / 2^12 / 2^13 / 2^14 / 2^15 points took 9.1 / 7.2
+// / 6.7 / 7.0 / 8.8 ms (512 integrals, 2-16 dimensions, 1e4..1e6 points, 5
+// iterations), 30 / 24 / 20 / 19 / 19 ms (1e4..1e7 points, 3 iterations) and
+// 30 / 23 / 21 / 24 / 31 ms (96 served requests to 1e7 points each).  At most
+// 32 tiles and 2^15 points take 6.95 and 18.5 ms in the two batches (16 and
+// 2^16, the rule before: 9.3 and 23.8); a serving round holds fewer
+// points for the same SMs, so its tiles stop at 2^13 (21.0 ms; before: 36.9).
+constexpr int kTileSplit = 32, kBatchTileCap = 1024, kServeTileCap = 256;
+
+// The order in which a launch hands its tiles out: the largest first (the
+// short ones then fill the queue's end), an integral's equal tiles
+// together, so that a CTA that takes several stages the integral once.
+static void order_tiles(Tile *first, Tile *last)
+{
+    std::stable_sort(first, last, [](const Tile &x, const Tile &y) { return x.nblk > y.nblk; });
+}
+
+// The device memory of one integral of a batch or a server: state, FP64
+// grid and the FP32 grid table, each on a 256-byte boundary.  (Their passes
+// leave the histogram as partial rows, so they need no BatchItem::H.)
+static size_t round256(size_t x) { return (x + 255) & ~(size_t)255; }
+static size_t item_bytes(int ndim, int N)
+{
+    return round256(sizeof(DevState)) + round256((size_t)ndim * (N + 1) * sizeof(double)) +
+           round256((size_t)ndim * N * sizeof(float2));
+}
+static void place_item(BatchItem *it, char *p, int ndim, int N)
+{
+    it->st = (DevState *)p;
+    p += round256(sizeof(DevState));
+    it->edges = (double *)p;
+    p += round256((size_t)ndim * (N + 1) * sizeof(double));
+    it->ew32 = (float2 *)p;
+    it->H = nullptr;
 }
 
 // A set of integrals run together: per iteration one persistent sampling
@@ -1573,8 +1609,9 @@ struct cv_batch {
     std::vector<cv_spec> specs;
     std::vector<int> jmax;                       // iterations of each integral
     std::vector<long long> n0;                   // first iteration size
-    void *mem = nullptr;                         // states, grids, histograms, logs
-    std::vector<double *> edges, log_I, log_var; // per integral (device)
+    void *mem = nullptr;                         // states, grids, grid tables, logs
+    std::vector<DevState *> states;              // per integral (device)
+    std::vector<double *> edges, log_I, log_var;
     std::vector<int> log_cap;                    // iterations each log holds
     BatchItem *d_items = nullptr;
     CombineArgs *d_cargs = nullptr;
@@ -1587,8 +1624,8 @@ struct cv_batch {
     // dimension classes: slots per axis, persistent grid
     struct Class { int ndim; bool pow2; int stride; int grid; };
     std::vector<Class> classes;
-    int tile_cap = 2048;                         // largest tile, in 32-point blocks
-    int tile_split = 16;                         // an iteration's tiles (at most), below the cap
+    int tile_cap = kBatchTileCap;                // largest tile, in 32-point blocks
+    int tile_split = kTileSplit;                 // an iteration's tiles (at most), below the cap
     int tile_fixed = 0;                          // CUBAGPU_TILE: every tile this size
     std::vector<int> item_class;
     // launch plan: per iteration, per class: tile offset and count, counter index
@@ -1684,6 +1721,7 @@ static int batch_build_tiles(cv_batch *B, int only_first_iteration)
                     t.item = i;
                     t.nblk = (int)(qb - q < (unsigned long long)TB ? qb - q : (unsigned long long)TB);
                     t.q0 = q;
+                    t.st = B->states[i];
                     t.row = (int)(tiles.size() - it0);
                     t.hoff = (unsigned)hf;
                     hf += (size_t)tp.stride;
@@ -1692,6 +1730,7 @@ static int batch_build_tiles(cv_batch *B, int only_first_iteration)
                 }
             }
             const int nt = (int)tiles.size() - off;
+            order_tiles(tiles.data() + off, tiles.data() + tiles.size());
             if (nt > 0) B->plan.push_back({j, (int)c, off, nt, counter++});
         }
         rows_max = std::max(rows_max, tiles.size() - it0);
@@ -1828,8 +1867,7 @@ extern "C" int cv_batch_create(cv_ctx *ctx, int count, const cv_spec *specs, cv_
     B->jmax.resize(count);
     B->n0.resize(count);
     B->item_class.resize(count);
-    // per-integral device memory: state, grid, histogram
-    const size_t sz_state = (sizeof(DevState) + 255) & ~(size_t)255;
+    // per-integral device memory: state, grid, grid table, log
     std::vector<size_t> off(count);
     size_t total = 0;
     for (int i = 0; i < count; ++i) {
@@ -1840,9 +1878,7 @@ extern "C" int cv_batch_create(cv_ctx *ctx, int count, const cv_spec *specs, cv_
         B->J = B->J > B->jmax[i] ? B->J : B->jmax[i];
         off[i] = total;
         const size_t lcap = (size_t)(B->jmax[i] < kLogCap ? B->jmax[i] : kLogCap);
-        total += sz_state + ((((size_t)ndim * (N + 1) * sizeof(double)) + 255) & ~(size_t)255) +
-                 ((((size_t)ndim * N * sizeof(double)) + 255) & ~(size_t)255) +
-                 ((2 * lcap * CV_MAX_COMP * sizeof(double) + 255) & ~(size_t)255);
+        total += item_bytes(ndim, N) + ((2 * lcap * CV_MAX_COMP * sizeof(double) + 255) & ~(size_t)255);
         // (the map's form decides the kernel: powers of two from 32 bins)
         const bool p2 = make_map(N, ndim, false).pow2 != 0;
         int c = -1;
@@ -1900,11 +1936,10 @@ extern "C" int cv_batch_create(cv_ctx *ctx, int count, const cv_spec *specs, cv_
         it.a.map = make_map(N, ndim, false);
         it.a.map.priv = it.a.map.pow2;  // every warp has its own histogram
         set_generator(&it.a, ndim, sp.flags, sp.seed);
-        it.st = (DevState *)p;
-        it.edges = (double *)(p + sz_state);
-        it.H = (double *)(p + sz_state + ((((size_t)ndim * (N + 1) * sizeof(double)) + 255) & ~(size_t)255));
+        place_item(&it, p, ndim, N);
         const int lcap = B->jmax[i] < kLogCap ? B->jmax[i] : kLogCap;
-        double *logs = it.H + (((((size_t)ndim * N * sizeof(double)) + 255) & ~(size_t)255) / sizeof(double));
+        double *logs = (double *)(p + item_bytes(ndim, N));
+        B->states.push_back(it.st);
         B->edges.push_back(it.edges);
         B->log_I.push_back(logs);
         B->log_var.push_back(logs + (size_t)lcap * CV_MAX_COMP);
@@ -2175,13 +2210,7 @@ private:
     std::map<size_t, size_t> free_;
 };
 
-size_t request_bytes(const cv_spec &sp)
-{
-    const size_t st = (sizeof(DevState) + 255) & ~(size_t)255;
-    const size_t e = (((size_t)sp.g.ndim * (sp.nbins + 1) * sizeof(double)) + 255) & ~(size_t)255;
-    const size_t h = (((size_t)sp.g.ndim * sp.nbins * sizeof(double)) + 255) & ~(size_t)255;
-    return st + e + h;
-}
+size_t request_bytes(const cv_spec &sp) { return item_bytes(sp.g.ndim, sp.nbins); }
 
 struct Request {
     uint64_t id;
@@ -2273,7 +2302,6 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
     const auto t0 = Clock::now();
     CV_CUDA(ctx, cudaEventRecord(S->ev_t0, S->stream));
     // descriptors of newly admitted requests
-    const size_t sz_state = (sizeof(DevState) + 255) & ~(size_t)255;
     for (const Request &r : live) {
         if (std::find(fresh.begin(), fresh.end(), r.slot) == fresh.end()) continue;
         const cv_spec &sp = r.spec;
@@ -2287,9 +2315,7 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
         it.a.map = make_map(N, ndim, false);
         it.a.map.priv = it.a.map.pow2;  // every warp has its own histogram
         set_generator(&it.a, ndim, sp.flags, sp.seed);
-        it.st = (DevState *)p;
-        it.edges = (double *)(p + sz_state);
-        it.H = (double *)(p + sz_state + ((((size_t)ndim * (N + 1) * sizeof(double)) + 255) & ~(size_t)255));
+        place_item(&it, p, ndim, N);
         CombineArgs ca = {};
         ca.st = it.st;
         ca.ncomp = sp.g.ncomp;
@@ -2333,13 +2359,14 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
         const unsigned long long s = r.next_index;
         const unsigned long long n = (unsigned long long)(r.spec.nstart + (long long)r.j * r.spec.nincrease);
         const long long tb = S->opts.tile_points > 0 ? std::max(1, S->opts.tile_points / 32)
-                                                     : tile_blocks_for((long long)n, 2048);
+                                                     : tile_blocks_for((long long)n, kServeTileCap, kTileSplit);
         const unsigned long long qa = (s >> 5) & ~1ull, qb = (s + n + 31) >> 5;
         for (unsigned long long q = qa; q < qb; q += (unsigned long long)tb) {
             Tile t;
             t.item = r.slot;
             t.nblk = (int)std::min<unsigned long long>(qb - q, (unsigned long long)tb);
             t.q0 = q;
+            t.st = (const DevState *)((const char *)S->arena_mem + r.off);
             c->tiles.push_back(t);
         }
         round_samples += (int64_t)n;
@@ -2368,6 +2395,13 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
         t.hoff = (unsigned)hf;
         hf += stride;
         ++tp.count;
+    }
+    {
+        Tile *t = all.data();
+        for (const Cls &c : cls) {
+            order_tiles(t, t + c.tiles.size());
+            t += c.tiles.size();
+        }
     }
     if (hf > 0xffffffffull) return fail_msg(ctx, CV_ENOMEM, "tile partials beyond 2^32 floats per round");
     {
@@ -3066,6 +3100,7 @@ struct SuaveMem {
     int grid = 0;               // persistent sampling grid
     int tile_cap = 0;           // tiles one pass may queue
     BatchItem *d_items = nullptr;  // [max_regions]: region k is item k
+    DevState *d_state = nullptr;   // [max_regions]
     int *d_counter = nullptr;
     char *d_stage = nullptr, *h_stage = nullptr;  // entries, tiles, axes of a pass
     double *dh_edges = nullptr, *dh_S = nullptr, *dh_fluct = nullptr;  // device addresses of the mirrors
@@ -3178,6 +3213,7 @@ int suave_pass_batched(cv_ctx *ctx, const cv_genz *g, int N, long long nnew, con
             T[nt].item = list[(size_t)i];
             T[nt].nblk = (int)(qb - q < (unsigned long long)TB ? qb - q : (unsigned long long)TB);
             T[nt].q0 = q;
+            T[nt].st = m.d_state + list[(size_t)i];
             ++nt;
         }
     }
@@ -3415,7 +3451,7 @@ int suave_batched_setup(cv_ctx *ctx, const cv_genz *g, int N, int flags, uint64_
     m.dh_S = m.dh_edges + (m.h_S - m.h_edges);
     m.dh_fluct = m.dh_edges + (m.h_fluct - m.h_edges);
     m.d_items = reinterpret_cast<BatchItem *>(d);
-    DevState *st = reinterpret_cast<DevState *>(d + sz_items);
+    DevState *st = m.d_state = reinterpret_cast<DevState *>(d + sz_items);
     m.d_stage = d + sz_items + sz_state;
     m.d_counter = reinterpret_cast<int *>(m.d_stage + sz_stage);
     m.h_stage = static_cast<char *>(*hstage);

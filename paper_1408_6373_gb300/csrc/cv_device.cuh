@@ -1240,6 +1240,15 @@ __device__ __forceinline__ void batch_steps(const SampleArgs<float> &A, const Sm
 // histogram): the sums of a tile never depend on which CTA ran it or on
 // what else was in the queue, and the rows are added in tile order, so an
 // integral gives the same result alone and in any mix, bit for bit.
+//
+// What a tile costs besides its points bounds how small tiles can be, and
+// small tiles are what keeps the queue's tail short.  So the chain of
+// dependent loads between tiles is taken off the path: the next tile is
+// claimed when a warp's points are done and its description arrives while
+// the copies are flushed (claiming earlier would hold a tile back from
+// idle CTAs); the grid comes as the table the refinement staged, not as
+// FP64 edges to convert (5 FP64 operations an entry, 2 a clock per SM);
+// and the flush moves four slots a time, in slot order.
 template <int NDIM, bool POW2>
 __global__ void __launch_bounds__(kBlock, (kMinBlocks<NDIM, float>))
 k_batch_sample(const BatchSampleArgs B)
@@ -1251,6 +1260,11 @@ k_batch_sample(const BatchSampleArgs B)
     sm.ew = align_table(smem_raw, stride);
     float *hist = reinterpret_cast<float *>(sm.ew + NDIM * stride);  // [kWarpsPerBlock][NDIM][stride]
     __shared__ __align__(16) SampleArgs<float> A;
+    // the tile in hand, in the place of the staged copy's part_* members
+    // (unused here): the shared memory left for ndim x nbins stays what it was
+    static_assert(sizeof(Tile) <= 32, "a tile fits the part_* members");
+    Tile &s_desc = *reinterpret_cast<Tile *>(&A.part_S);
+    const int staged = (int)((reinterpret_cast<char *>(&A.part_S) - reinterpret_cast<char *>(&A)) / sizeof(int));
     __shared__ int s_tile;
     __shared__ double red[kWarpsPerBlock][2 * CV_MAX_COMP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1258,91 +1272,139 @@ k_batch_sample(const BatchSampleArgs B)
     sm.h = hist + warp * hsize;
     for (int i = threadIdx.x; i < kWarpsPerBlock * hsize; i += blockDim.x) hist[i] = 0.0f;
     int cur = -1;
+    if (threadIdx.x == 0) {
+        const int t = atomicAdd(B.counter, 1);
+        s_tile = t;
+        if (t < B.ntiles) s_desc = B.tiles[t];
+    }
     for (;;) {
-        if (threadIdx.x == 0) s_tile = atomicAdd(B.counter, 1);
         __syncthreads();
-        const int t = s_tile;
-        if (t >= B.ntiles) break;
-        const Tile tile = B.tiles[t];
+        if (s_tile >= B.ntiles) break;
+        const Tile tile = s_desc;
+        const int stopped = *(volatile const int *)&tile.st->stopped;
+        const unsigned long long start = tile.st->next_index;
+        const unsigned long long end = start + (unsigned long long)tile.st->n_cur;
         const BatchItem &it = B.items[tile.item];
-        if (*(volatile const int *)&it.st->stopped) {
-            __syncthreads();
-            continue;
-        }
-        if (tile.item != cur) {
+        if (!stopped && tile.item != cur) {
             // stage the integral's parameters and grid
             const int *src = reinterpret_cast<const int *>(&it.a);
             int *dst = reinterpret_cast<int *>(&A);
-            for (int i = threadIdx.x; i < (int)(sizeof(SampleArgs<float>) / sizeof(int)); i += blockDim.x)
-                dst[i] = src[i];
+            for (int i = threadIdx.x; i < staged; i += blockDim.x) dst[i] = src[i];
+            const float2 *ew32 = it.ew32;
+            const int n = it.a.nbins;
+            if (ew32 && n == stride) {
+                // (even stride: the POW2 classes and any even bin count)
+                if (stride % 2 == 0) {
+                    const float4 *g4 = reinterpret_cast<const float4 *>(ew32);
+                    float4 *t4 = reinterpret_cast<float4 *>(sm.ew);
+                    for (int i = threadIdx.x; i < NDIM * stride / 2; i += blockDim.x) t4[i] = g4[i];
+                } else {
+                    for (int i = threadIdx.x; i < NDIM * stride; i += blockDim.x) sm.ew[i] = ew32[i];
+                }
+            } else if (ew32) {
+                for (int i = threadIdx.x; i < NDIM * n; i += blockDim.x) {
+                    const int d = i / n;
+                    sm.ew[d * stride + (i - d * n)] = ew32[i];
+                }
+            } else {
+                stage_grid_f32(sm.ew, NDIM, n, stride, it.edges, it.a.map);
+            }
+            cur = tile.item;
             __syncthreads();
-            stage_grid_f32(sm.ew, NDIM, A.nbins, stride, it.edges, A.map);
             // (the grid and histogram bases are multiples of 8 stride and
             // 4 stride, stride a multiple of this integral's N)
             set_addresses(sm, POW2 ? A.map.L : 0);
-            cur = tile.item;
-            __syncthreads();
         }
-        const unsigned long long start = it.st->next_index;
-        const unsigned long long end = start + (unsigned long long)it.st->n_cur;
         Acc<float> s1[CV_MAX_COMP], s2[CV_MAX_COMP];
-        // (an even share, so that warps start on even blocks of an even tile)
-        const unsigned per = ((((unsigned)tile.nblk + kWarpsPerBlock - 1) / kWarpsPerBlock) + 1u) & ~1u;
-        const unsigned long long w0 = tile.q0 + (unsigned long long)warp * per;
-        const unsigned long long w1 = min(w0 + per, tile.q0 + (unsigned long long)tile.nblk);
-        const int hmode = A.map.priv ? kHistWarpPlain : kHistWarpAtomic;
-        if (w0 < w1) {
-            unsigned X[NDIM];
-            sobol_skip<NDIM, unsigned>(X, w0, lane, POW2 ? A.map.li : 0);
-            if (A.gen == kGenScrambled) {
+        if (!stopped) {
+            // (an even share, so that warps start on even blocks of an even tile)
+            const unsigned per = ((((unsigned)tile.nblk + kWarpsPerBlock - 1) / kWarpsPerBlock) + 1u) & ~1u;
+            const unsigned long long w0 = tile.q0 + (unsigned long long)warp * per;
+            const unsigned long long w1 = min(w0 + per, tile.q0 + (unsigned long long)tile.nblk);
+            const int hmode = A.map.priv ? kHistWarpPlain : kHistWarpAtomic;
+            if (w0 < w1) {
+                unsigned X[NDIM];
+                sobol_skip<NDIM, unsigned>(X, w0, lane, POW2 ? A.map.li : 0);
+                if (A.gen == kGenScrambled) {
 #pragma unroll
-                for (int d = 0; d < NDIM; ++d) X[d] ^= (unsigned)A.shift[d];
+                    for (int d = 0; d < NDIM; ++d) X[d] ^= (unsigned)A.shift[d];
+                }
+                const bool interior = (w0 * 32ull >= start) && (w1 * 32ull <= end) && !((w0 | w1) & 1ull);
+                if (interior)
+                    batch_steps<NDIM, POW2, false>(A, sm, X, w0, (unsigned)(w1 - w0), start, end, lane, hmode, s1, s2);
+                else
+                    batch_steps<NDIM, POW2, true>(A, sm, X, w0, (unsigned)(w1 - w0), start, end, lane, hmode, s1, s2);
             }
-            const bool interior = (w0 * 32ull >= start) && (w1 * 32ull <= end) && !((w0 | w1) & 1ull);
-            if (interior)
-                batch_steps<NDIM, POW2, false>(A, sm, X, w0, (unsigned)(w1 - w0), start, end, lane, hmode, s1, s2);
-            else
-                batch_steps<NDIM, POW2, true>(A, sm, X, w0, (unsigned)(w1 - w0), start, end, lane, hmode, s1, s2);
         }
-        const int ncomp = A.g.ncomp;
+        int next = 0;
+        if (threadIdx.x == 0) next = atomicAdd(B.counter, 1);
+        if (!stopped) {
+            const int ncomp = A.g.ncomp;
 #pragma unroll
-        for (int c = 0; c < CV_MAX_COMP; ++c) {
-            if (c < ncomp) {
-                const double a = warp_total(s1[c]);
-                const double b = warp_total(s2[c]);
-                if (lane == 0) {
-                    red[warp][2 * c] = a;
-                    red[warp][2 * c + 1] = b;
+            for (int c = 0; c < CV_MAX_COMP; ++c) {
+                if (c < ncomp) {
+                    const double a = warp_total(s1[c]);
+                    const double b = warp_total(s2[c]);
+                    if (lane == 0) {
+                        red[warp][2 * c] = a;
+                        red[warp][2 * c + 1] = b;
+                    }
                 }
             }
         }
-        __syncthreads();
-        // the tile's sums and histogram: its partial rows (part_S), else
-        // FP64 atomics into the integral's state
-        if (threadIdx.x < 2 * ncomp) {
-            double v = 0.0;
-            for (int w = 0; w < kWarpsPerBlock; ++w) v += red[w][threadIdx.x];
-            const int c = threadIdx.x >> 1;
-            if (B.part_S) B.part_S[(size_t)tile.row * (2 * CV_MAX_COMP) + threadIdx.x] = v;
-            else atomicAdd((threadIdx.x & 1) ? &it.st->S2[c] : &it.st->S1[c], v);
-        }
-        // (warp copies summed in warp order, then cleared)
-        const int N = A.nbins;
-        float *ph = B.part_S ? B.part_H + tile.hoff : nullptr;
-        for (int idx = threadIdx.x; idx < NDIM * N; idx += blockDim.x) {
-            const int d = idx / N, sl = idx - d * N;  // (by slot: conflict-free)
-            const int p = d * stride + sl;
-            float v = 0.0f;
-#pragma unroll
-            for (int w = 0; w < kWarpsPerBlock; ++w) {
-                float &e = hist[w * hsize + p];
-                v += e;
-                e = 0.0f;
+        __syncthreads();  // (every thread has read s_tile and s_desc)
+        Tile desc;
+        if (threadIdx.x == 0 && next < B.ntiles) desc = B.tiles[next];
+        if (!stopped) {
+            const int ncomp = A.g.ncomp;
+            // the tile's sums and histogram: its partial rows (part_S), else
+            // FP64 atomics into the integral's state
+            if (threadIdx.x < 2 * ncomp) {
+                double v = 0.0;
+                for (int w = 0; w < kWarpsPerBlock; ++w) v += red[w][threadIdx.x];
+                const int c = threadIdx.x >> 1;
+                if (B.part_S) B.part_S[(size_t)tile.row * (2 * CV_MAX_COMP) + threadIdx.x] = v;
+                else atomicAdd((threadIdx.x & 1) ? &it.st->S2[c] : &it.st->S1[c], v);
             }
-            if (ph) ph[d * N + bin_of_slot(sl, A.map)] = v;
-            else if (v != 0.0f) atomicAdd(&it.H[d * N + bin_of_slot(sl, A.map)], (double)v);
+            // (warp copies summed in warp order, then cleared)
+            const int N = A.nbins;
+            float *ph = B.part_S ? B.part_H + tile.hoff : nullptr;
+            if (POW2 && ph && N == stride) {
+                // (N a multiple of 32: rows and copies are 16-byte aligned)
+                float4 *ph4 = reinterpret_cast<float4 *>(ph);
+                for (int i = threadIdx.x; i < hsize / 4; i += blockDim.x) {
+                    float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+                    for (int w = 0; w < kWarpsPerBlock; ++w) {
+                        float4 &e = reinterpret_cast<float4 *>(hist + w * hsize)[i];
+                        v.x += e.x;
+                        v.y += e.y;
+                        v.z += e.z;
+                        v.w += e.w;
+                        e = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    }
+                    ph4[i] = v;
+                }
+            } else {
+                for (int idx = threadIdx.x; idx < NDIM * N; idx += blockDim.x) {
+                    const int d = idx / N, sl = idx - d * N;  // (by slot: conflict-free)
+                    const int p = d * stride + sl;
+                    float v = 0.0f;
+#pragma unroll
+                    for (int w = 0; w < kWarpsPerBlock; ++w) {
+                        float &e = hist[w * hsize + p];
+                        v += e;
+                        e = 0.0f;
+                    }
+                    if (ph) ph[idx] = v;
+                    else if (v != 0.0f) atomicAdd(&it.H[d * N + bin_of_slot(sl, A.map)], (double)v);
+                }
+            }
         }
-        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_tile = next;
+            if (next < B.ntiles) s_desc = desc;
+        }
     }
 }
 

@@ -215,7 +215,9 @@ struct SampleArgs {
     // are summed per bin in block order by that kernel too (refinement, or
     // a reduction after a standalone pass).  Null: FP64 atomics, whose
     // order varies from run to run.
-    double *part_S;                 // [part_G][2 CV_MAX_COMP]
+    // (16-byte aligned: the batched kernel keeps a tile in its staged copy's
+    // place of these four)
+    alignas(16) double *part_S;     // [part_G][2 CV_MAX_COMP]
     void *part_H;                   // [part_G][ndim][nbins]
     unsigned *part_ticket;
     int part_G;
@@ -242,6 +244,7 @@ struct CombineArgs {
     int part_G;
     int part_nh;                    // ndim * nbins: values per block
     int part_f32;                   // partials are floats (FP32 pass)
+    int part_slots;                 // rows in slot order (slot_of_bin), else by bin
     // the pass's sum partials (SampleArgs::part_S of a launch without a
     // ticket), summed by the combination in block order; null: the pass
     // added them to S1, S2 itself
@@ -258,16 +261,23 @@ struct BatchItem {
     SampleArgs<float> a;            // parameters, map, nbins (pointers unused)
     DevState *st;
     double *edges;                  // [ndim][nbins+1]
-    double *H;                      // [ndim][nbins]
+    double *H;                      // [ndim][nbins]; null where every pass leaves partial rows
+    // the FP32 grid table of `edges` (SampleArgs::ew32's layout), 16-byte
+    // aligned, written by the reset and by each refinement; null: every
+    // tile's CTA converts the FP64 edges itself
+    float2 *ew32;
 };
 
 // A tile: nblk consecutive 32-point Sobol blocks of one integral's
 // iteration, starting at absolute block q0.  row, hoff: where the tile
 // leaves its sums and histogram when the launch reduces through partials.
-struct Tile {
+// st: the integral's state, so that a CTA reaches the stop flag and the
+// index range one load after the tile (32 bytes: two 16-byte loads).
+struct alignas(16) Tile {
     int item;
     int nblk;
     unsigned long long q0;
+    const DevState *st;
     int row;                        // row of BatchSampleArgs::part_S
     unsigned hoff;                  // first float of its [ndim][nbins] rows in part_H
 };
@@ -289,7 +299,7 @@ struct BatchSampleArgs {
     int stride;                     // slots per axis: the class's largest nbins
     int *counter;                   // next tile to take (zero before the launch)
     // Deterministic reduction (part_S non-null): tile t writes its sums to
-    // part_S[t.row][2 c + {0, 1}] and its histogram, by bin, to part_H +
+    // part_S[t.row][2 c + {0, 1}] and its histogram, by slot, to part_H +
     // t.hoff, no atomics; the batched refinement and combination add an
     // integral's rows in tile order.  Null: FP64 atomics into the
     // integral's state and histogram.

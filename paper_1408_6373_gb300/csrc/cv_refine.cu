@@ -182,7 +182,7 @@ __device__ __forceinline__ void sum_rows(const T *P, int G, size_t nh, int N,
     for (int i = 0; i < V; ++i) grp[r * N + q * V + i] = {s[i], c[i]};
 }
 
-__device__ void sum_parts_axis(const CombineArgs *pa, int d, int N, double *sH)
+__device__ void sum_parts_axis(const CombineArgs *pa, int d, int N, double *sH, const MapParams *map)
 {
     // R x N group sums, R N <= 4 blockDim (FP32), 2 blockDim (FP64)
     __shared__ __align__(16) unsigned char grp_raw[4096 * sizeof(float2)];
@@ -205,7 +205,9 @@ __device__ void sum_parts_axis(const CombineArgs *pa, int d, int N, double *sH)
                 kahan_add(s, c, g.x);
                 kahan_add(s, c, -g.y);
             }
-            sH[k] = (double)s - (double)c;
+            // (rows in slot order: the writer's stores are then contiguous,
+            // and one permuted store here costs nothing)
+            sH[pa->part_slots ? bin_of_slot(k, *map) : k] = (double)s - (double)c;
         }
     } else {
         double2 *grp = reinterpret_cast<double2 *>(grp_raw);
@@ -226,7 +228,7 @@ __device__ void sum_parts_axis(const CombineArgs *pa, int d, int N, double *sH)
 __device__ void refine_axis(int d, int N, double *H, double *edges, int zero_hist, float2 *ew32 = nullptr,
                             const MapParams *map = nullptr, const CombineArgs *pa = nullptr)
 {
-    double *Hd = H + (size_t)d * N;
+    double *Hd = H ? H + (size_t)d * N : nullptr;
     double *e = edges + (size_t)d * (N + 1);
     __shared__ double sH[CV_MAX_BINS], sq[CV_MAX_BINS];
     __shared__ double sC[CV_MAX_BINS + 1], se[CV_MAX_BINS + 1];
@@ -240,7 +242,7 @@ __device__ void refine_axis(int d, int N, double *H, double *edges, int zero_his
     const bool act = warp < nw;
     const double invN = __drcp_rn((double)N);  // (off the dependent chain)
 
-    if (pa && pa->part_H) sum_parts_axis(pa, d, N, sH);
+    if (pa && pa->part_H) sum_parts_axis(pa, d, N, sH, map);
     else if (k < N) sH[k] = Hd[k];
     for (int i = k; i <= N; i += blockDim.x) se[i] = e[i];
     __syncthreads();
@@ -559,7 +561,12 @@ __global__ void k_batch_reset(const BatchItem *items, const CombineArgs *cargs, 
         const int k = i % (N + 1);
         it.edges[i] = (double)k / (double)N;
     }
-    for (int i = threadIdx.x; i < ndim * N; i += blockDim.x) it.H[i] = 0.0;
+    if (it.H)
+        for (int i = threadIdx.x; i < ndim * N; i += blockDim.x) it.H[i] = 0.0;
+    if (it.ew32) {
+        __syncthreads();  // (the edges written above)
+        for (int d = 0; d < ndim; ++d) stage_axis(d, N, it.edges, it.ew32, it.a.map, threadIdx.x, blockDim.x);
+    }
     int *w = reinterpret_cast<int *>(it.st);
     for (int i = threadIdx.x; i < (int)(sizeof(DevState) / sizeof(int)); i += blockDim.x) w[i] = 0;
     __syncthreads();
@@ -583,9 +590,10 @@ __global__ void __launch_bounds__(256) k_batch_refine(const BatchItem *items, co
         pa.part_G = tp.count;
         pa.part_nh = tp.stride;
         pa.part_f32 = 1;
-        refine_axis(ax.y, it.a.nbins, it.H, it.edges, 1, nullptr, nullptr, &pa);
+        pa.part_slots = 1;
+        refine_axis(ax.y, it.a.nbins, it.H, it.edges, 0, it.ew32, &it.a.map, &pa);
     } else {
-        refine_axis(ax.y, it.a.nbins, it.H, it.edges, 1);
+        refine_axis(ax.y, it.a.nbins, it.H, it.edges, 1, it.ew32, &it.a.map);
     }
 }
 
