@@ -464,25 +464,39 @@ static int occupancy(cv_ctx *ctx, int ndim, int nbins, bool fp64, int *occ)
     return CV_OK;
 }
 
-// Blocks for a pass over n points: about 16 32-point blocks per warp, at
-// most one full wave of resident CTAs.  A pass too small to fill that wave
-// spreads over more warps instead (down to 2 blocks each): its time is the
-// dependent arithmetic of one warp's blocks (FP64 especially), not issue.
-static int sample_grid(cv_ctx *ctx, int occ, long long n)
+// Blocks for a pass over n points: as many CTAs per SM as leave every warp
+// about ten 32-point blocks, at most one full wave of resident CTAs; a pass
+// too small for one CTA on every SM spreads over the SMs, six blocks per
+// CTA.  A CTA costs its prologue (the grid table, the histogram copies) and
+// a partial row that the refinement adds, so more CTAs than the points need
+// are not free; us per iteration (6 dimensions, 2 components, 64 bins), on
+// 76 / 152 / 304 / 456 CTAs: 16.0 / 15.5 / 16.4 / 17.4 for 3e4 points,
+// 23.0 / 19.2 / 19.1 / 21.0 for 3e5, 44 / 29.0 / 24.8 / 26.2 for 1e6,
+// 104 / 59 / 41.7 / 39.0 for 3e6.  An FP64 pass takes a block for each of
+// four warps of a CTA: its time is the SM's FP64 lanes, which all its warps
+// share (and the refinement's is the rows it adds, so not one warp per CTA):
+// 3 dimensions, 50 bins, 1e4 points 17.2 us an iteration, 18.8 with one or
+// two and 18.5 with eight.
+static int sample_grid(cv_ctx *ctx, int occ, long long n, bool fp64)
+{
+    const long long nblk = (n + 63) / 32, sms = ctx->sms;
+    const long long small = fp64 ? (nblk + 3) / 4 : (nblk + 5) / 6;
+    if (small < sms) return small < 1 ? 1 : (int)small;
+    const long long per_sm = nblk / (sms * kWarpsPerBlock * 10);
+    return (int)(sms * std::min<long long>(std::max<long long>(per_sm, 1), occ));
+}
+
+// Blocks for a materialised pass over n points (bound by HBM, so a full wave
+// as soon as there are about 16 32-point blocks per warp, and down to 2 below
+// that).
+static int mat_grid(cv_ctx *ctx, int occ, long long n)
 {
     const long long nblk = (n + 63) / 32;
     const long long cap = (long long)ctx->sms * occ;
     long long want = (nblk + (long long)kWarpsPerBlock * 16 - 1) / ((long long)kWarpsPerBlock * 16);
-    if (want < cap) {
-        want = (nblk + (long long)kWarpsPerBlock * 2 - 1) / ((long long)kWarpsPerBlock * 2);
-        if (want > cap) want = cap;
-    }
-    if (want > cap) want = cap;
-    if (want < 1) want = 1;
-    return (int)want;
+    if (want < cap) want = (nblk + (long long)kWarpsPerBlock * 2 - 1) / ((long long)kWarpsPerBlock * 2);
+    return (int)std::max<long long>(1, std::min(want, cap));
 }
-
-
 
 // Per-block partials of a deterministic pass, in one device block laid out
 // as [ticket (256 bytes)][S: G_cap x 2 CV_MAX_COMP doubles][H: G_cap x ndim
@@ -520,14 +534,14 @@ static int pass_grid(cv_ctx *ctx, const cv_genz *g, int nbins, int flags, long l
             JitKernel k;
             std::string err;
             if (jit_sample_kernel(ctx->device, a, g->ndim, a.map.pow2 != 0, min_blocks_f32(g->ndim), &k, &err) == 0) {
-                *grid = sample_grid(ctx, k.occ, n_grid);
+                *grid = sample_grid(ctx, k.occ, n_grid, false);
                 return CV_OK;
             }
         }
     }
     int occ = 0, rc = occupancy(ctx, g->ndim, nbins, sizeof(Real) == 8, &occ);
     if (rc) return rc;
-    *grid = sample_grid(ctx, occ, n_grid);
+    *grid = sample_grid(ctx, occ, n_grid, sizeof(Real) == 8);
     return CV_OK;
 }
 
@@ -543,7 +557,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
     memset(&a, 0, sizeof(a));
     fill_params<Real>(g, &a.g);
     a.nbins = nbins;
-    a.chunk_min = 2;
+    a.chunk_min = sizeof(Real) == 8 ? 1 : 2;
     a.map = make_map(nbins, g->ndim, sizeof(Real) == 8);
     set_generator(&a, g->ndim, flags, seed);
     const bool jit = (flags & CV_JIT) != 0;
@@ -568,7 +582,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
             JitKernel k;
             std::string err;
             if (jit_sample_kernel(ctx->device, a, g->ndim, a.map.pow2 != 0, min_blocks_f32(g->ndim), &k, &err) == 0) {
-                const int grid = sample_grid(ctx, k.occ, n_grid);
+                const int grid = sample_grid(ctx, k.occ, n_grid, false);
                 use_parts(grid);
                 const int tk = timer_begin(ctx);
                 cudaError_t e = launch_jit_sample(k, a, grid, ctx->stream);
@@ -582,7 +596,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
     }
     int occ = 0, rc = occupancy(ctx, g->ndim, nbins, sizeof(Real) == 8, &occ);
     if (rc) return rc;
-    const int grid = sample_grid(ctx, occ, n_grid);
+    const int grid = sample_grid(ctx, occ, n_grid, sizeof(Real) == 8);
     use_parts(grid);
     const int tk = timer_begin(ctx);
     cudaError_t e = dispatch_sample<Real>(g->ndim, a, grid, ctx->stream);
@@ -1934,7 +1948,7 @@ extern "C" int cv_batch_create(cv_ctx *ctx, int count, const cv_spec *specs, cv_
         it.a.nbins = N;
         it.a.chunk_min = 4;
         it.a.map = make_map(N, ndim, false);
-        it.a.map.priv = it.a.map.pow2;  // every warp has its own histogram
+        it.a.map.priv = hist_phases(N);  // (every warp has its own histogram)
         set_generator(&it.a, ndim, sp.flags, sp.seed);
         place_item(&it, p, ndim, N);
         const int lcap = B->jmax[i] < kLogCap ? B->jmax[i] : kLogCap;
@@ -2313,7 +2327,7 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
         it.a.nbins = N;
         it.a.chunk_min = 4;
         it.a.map = make_map(N, ndim, false);
-        it.a.map.priv = it.a.map.pow2;  // every warp has its own histogram
+        it.a.map.priv = hist_phases(N);  // (every warp has its own histogram)
         set_generator(&it.a, ndim, sp.flags, sp.seed);
         place_item(&it, p, ndim, N);
         CombineArgs ca = {};
@@ -2922,7 +2936,7 @@ static int vegas_cb_run(cv_ctx *ctx, int ndim, int ncomp, cv_integrand_dev cb, v
     // histogram rows) before the next.
     PassParts pp;
     if (e == cudaSuccess) {
-        const int rc_p = ctx_parts(ctx, sample_grid(ctx, occ, tile), &pp);
+        const int rc_p = ctx_parts(ctx, mat_grid(ctx, occ, tile), &pp);
         if (rc_p) {
             cudaEventDestroy(ev_stop);
             return rc_p;
@@ -2935,7 +2949,7 @@ static int vegas_cb_run(cv_ctx *ctx, int ndim, int ncomp, cv_integrand_dev cb, v
         b.start = s0;
         b.n = m;
         // (the same grid as a fused pass: the kernels share its occupancy)
-        return dispatch_matpass<Real>(ndim, false, b, sample_grid(ctx, occ, m), s, &grid_used);
+        return dispatch_matpass<Real>(ndim, false, b, mat_grid(ctx, occ, m), s, &grid_used);
     };
     if (e == cudaSuccess && jmax > 0) e = store(start, sp.nstart < tile ? sp.nstart : tile);
     double *pp_S = nullptr;
@@ -2961,7 +2975,7 @@ static int vegas_cb_run(cv_ctx *ctx, int ndim, int ncomp, cv_integrand_dev cb, v
             parts_args(&pp, 0, &b.part_S, &b.part_H, &b.part_ticket);
             b.part_G = pp.G_cap;
             if (one_tile) b.part_ticket = nullptr;  // (the combination adds the sums)
-            e = dispatch_matpass<Real>(ndim, true, b, sample_grid(ctx, occ, m), s, &grid_used);
+            e = dispatch_matpass<Real>(ndim, true, b, mat_grid(ctx, occ, m), s, &grid_used);
             if (e == cudaSuccess && !one_tile)
                 e = launch_add_parts(b.part_H, grid_used, fp32 ? 1 : 0, nh, H, s);
         }
@@ -3466,7 +3480,7 @@ int suave_batched_setup(cv_ctx *ctx, const cv_genz *g, int N, int flags, uint64_
     proto.a.nbins = N;
     proto.a.chunk_min = 4;
     proto.a.map = make_map(N, ndim, false);
-    proto.a.map.priv = proto.a.map.pow2;  // every warp has its own histogram
+    proto.a.map.priv = hist_phases(N);  // (every warp has its own histogram)
     set_generator(&proto.a, ndim, flags, seed);
     for (int k = 0; k < max_regions; ++k) {
         items[(size_t)k] = proto;

@@ -190,20 +190,21 @@ __device__ __forceinline__ float ipow(float r)
     return acc;
 }
 
-// (h + l)^E for h + l carried to about twice binary32 precision: each
+// (h + l)^E for h + l carried to about twice the precision of T: each
 // product of pairs keeps its rounding error (FMA) and the cross terms,
 // (ah + al)(bh + bl) = ah bh + [err(ah bh) + al bh + ah bl] + al bl, the
 // last term below the pair's precision.  Returns the high part, the low
 // part in lo.
-__device__ __forceinline__ void mul_df(float ah, float al, float bh, float bl, float &h, float &l)
+template <typename T>
+__device__ __forceinline__ void mul_df(T ah, T al, T bh, T bl, T &h, T &l)
 {
     h = ah * bh;
-    l = __fmaf_rn(ah, bl, __fmaf_rn(al, bh, __fmaf_rn(ah, bh, -h)));
+    l = fma_rn(ah, bl, fma_rn(al, bh, fma_rn(ah, bh, -h)));
 }
-template <int E>
-__device__ __forceinline__ float ipow_df(float h, float l, float &lo)
+template <int E, typename T>
+__device__ __forceinline__ T ipow_df(T h, T l, T &lo)
 {
-    float ah = 1.0f, al = 0.0f, bh = h, bl = l;
+    T ah = T(1), al = T(0), bh = h, bl = l;
     int e = E;
     bool first = true;
 #pragma unroll
@@ -424,16 +425,34 @@ __device__ __forceinline__ double genz_f64(const GenzParams<double> &g, const do
         for (int d = 0; d < NDIM; ++d) s = __fma_rn(I::template p0<C>(g, d), x[d], s);
         return cos(I::template q0<C>(g) + s);
     case CV_PRODUCT_PEAK:
+        // prod 1 / (1/a^2 + (x - u)^2): one reciprocal for up to eight axes
+        // (a product of eight denominators stays in range wherever the
+        // product of their reciprocals does) and half the roundings
 #pragma unroll
-        for (int d = 0; d < NDIM; ++d) {
-            const double dx = x[d] - I::template p1<C>(g, d);
-            P *= 1.0 / __fma_rn(dx, dx, I::template p0<C>(g, d));
+        for (int d0 = 0; d0 < NDIM; d0 += 8) {
+            double q = 1.0;
+#pragma unroll
+            for (int d = d0; d < d0 + 8 && d < NDIM; ++d) {
+                const double dx = x[d] - I::template p1<C>(g, d);
+                q *= __fma_rn(dx, dx, I::template p0<C>(g, d));
+            }
+            P *= __drcp_rn(q);
         }
         return P;
-    case CV_CORNER_PEAK:
+    case CV_CORNER_PEAK: {
+        // s^-(NDIM+1) as a product of pairs (high and low parts): the
+        // reciprocal's residual is its low part, so the result is good to an
+        // ulp, as pow's was, in ~4 FP64 operations per multiplication
+        // (pow takes ~150, half of an evaluation of four components)
 #pragma unroll
         for (int d = 0; d < NDIM; ++d) s = __fma_rn(I::template p0<C>(g, d), x[d], s);
-        return pow(1.0 + s, -(double)(NDIM + 1));
+        s += 1.0;
+        const double r = __drcp_rn(s);
+        const double w = r > 0.0 ? __fma_rn(-s, r, 1.0) : 0.0;  // (s may be infinite)
+        double fl;
+        const double fh = ipow_df<NDIM + 1>(r, r * w, fl);
+        return fh + fl;
+    }
     case CV_GAUSSIAN:
 #pragma unroll
         for (int d = 0; d < NDIM; ++d) {
@@ -524,10 +543,9 @@ __device__ __forceinline__ double warp_total(const Acc<double> &a)
 }
 
 // ------------------------------------------------------------ sampling steps
-// Shared-memory views of one block.  FP64: every axis owns a stride of
-// CV_MAX_BINS slots.  FP32: `stride` entries per axis (nbins, or the batch
-// class's largest nbins), a compile-time constant in the specialised kernel.
-constexpr int kStride = CV_MAX_BINS;
+// Shared-memory views of one block: `stride` entries per axis (nbins, or
+// the batch class's largest nbins), a compile-time constant in the
+// specialised kernel.
 
 template <typename Real> struct Smem;
 template <> struct Smem<float> {
@@ -542,15 +560,17 @@ template <> struct Smem<float> {
 };
 template <> struct Smem<double> {
     double2 *ew;       // [NDIM][stride] {e_k, w_k}
-    double *h;         // [NDIM][hs]
-    int stride, hs;
+    double *h;         // the histogram copy this warp updates: its own [NDIM][stride], or the block's
+    int stride;        // nbins
+    double n8, nr;     // N^8 and N^(NDIM mod 8): the factors of J (jacobian_scale)
 };
 
-// How a block accumulates its FP32 f^2 histogram: one copy per warp,
-// updated with plain loads and stores when the 32 lanes' bins are distinct
-// (N = 2^L >= 32) or with shared atomics otherwise; or one block copy with
-// shared atomics.
-enum { kHistWarpPlain = 0, kHistWarpAtomic = 1, kHistBlock = 2 };
+// How a block accumulates its f^2 histogram: one copy per warp, updated
+// with plain loads and stores when the 32 lanes' bins are distinct
+// (N = 2^L >= 32), or in MapParams::priv such steps over the lanes whose
+// strata agree (other N); or one block copy with shared atomics (copies
+// that do not fit, and pseudo-random points).
+enum { kHistWarpPlain = 0, kHistWarpPhased = 1, kHistBlock = 2 };
 
 // The shared-window addresses of a block's FP32 grid and histogram copy
 // (L = log2 N of the power-of-two map, else 0).
@@ -634,17 +654,36 @@ __device__ __forceinline__ float map_f32(unsigned X, int d, int N, const MapPara
     }
 }
 
+// t 2^-52 for t < 2^52, from the bits: an FP64 instruction costs as many
+// issue slots as ~60 integer ones here (2 FP64 lanes per SM), so the usual
+// (1 + t 2^-52) - 1 is the dearer way.
+__device__ __forceinline__ double frac52(unsigned long long t)
+{
+    const int lz = __clzll((long long)t);
+    const unsigned long long v = (t << (lz - 11)) + ((unsigned long long)(1033 - lz) << 52);
+    return __longlong_as_double((long long)(t ? v : 0ull));
+}
+
+// N^k, k <= 8: exact for powers of two, else rounded once.
+__device__ __forceinline__ double jacobian_scale(int N, int k)
+{
+    if (N == CV_MAX_BINS && k == 8) return 18446744073709551616.0;
+    unsigned long long p = 1;
+    for (int i = 0; i < k; ++i) p *= (unsigned long long)N;
+    return (double)p;
+}
+
+// Map one FP64 coordinate; J collects the widths (the factors N^8 are
+// applied every eight axes by the caller).
 __device__ __forceinline__ double map_f64(unsigned long long X, int d, int N,
                                           const Smem<double> &sm, double &J, int &slot)
 {
     const unsigned long long t = (X >> 12) * (unsigned long long)N;  // < 2^60
-    const double frac = __longlong_as_double((long long)(0x3ff0000000000000ull |
-                                                         (t & 0xfffffffffffffull))) - 1.0;
     const int p = (int)(t >> 52);
     const double2 ew = sm.ew[d * sm.stride + p];
-    J = J * ((double)N * ew.y);
+    J *= ew.y;
     slot = p;
-    return __fma_rn(ew.y, frac, ew.x);
+    return __fma_rn(ew.y, frac52(t & 0xfffffffffffffull), ew.x);
 }
 
 template <typename Real> struct Word;
@@ -753,8 +792,9 @@ __device__ __forceinline__ void sample_block(const SampleArgs<float> &A, const S
     if (EDGE && !valid) J = 0.0f;  // (f is finite at every point of the block)
     // the f^2 histogram needs component 0 only: updated before the other
     // components are evaluated, so the bins' offsets are dead by then
+    // (an invalid point's J is 0: it adds nothing to its bins)
     const float v0 = J * f[0];
-    if (!EDGE || valid) {
+    {
         const float h = v0 * v0;
         // the bin's float in the histogram copy: one funnel shift of the
         // word (power-of-two map), or slot * 4 (general map)
@@ -773,9 +813,21 @@ __device__ __forceinline__ void sample_block(const SampleArgs<float> &A, const S
 #pragma unroll
                 for (int d = d0; d < d0 + kHistBatch && d < NDIM; ++d) sts_f(haddr(d), hv[d - d0] + h);
             }
-        } else {
+        } else if (POW2 || hmode != kHistWarpPhased) {
 #pragma unroll
             for (int d = 0; d < NDIM; ++d) reds_add_f(haddr(d), h);
+        }
+        if (!POW2 && hmode == kHistWarpPhased) {
+            // (the top five bits of an unmapped word are its stratum; one
+            // axis at a time: batched as above, the batched kernel spills)
+            const unsigned mask = (unsigned)(A.map.priv - 1) << 27;
+#pragma unroll 1
+            for (unsigned ph = 0; ph <= mask; ph += 1u << 27) {
+#pragma unroll
+                for (int d = 0; d < NDIM; ++d)
+                    if ((X[d] & mask) == ph) sts_f(haddr(d), lds_f(haddr(d)) + h);
+                __syncwarp();
+            }
         }
     }
     if constexpr (I::kMode != 2) {
@@ -815,7 +867,11 @@ __device__ __forceinline__ void sample_block(const SampleArgs<double> &A, const 
     int slot[NDIM];
     double J = 1.0;
 #pragma unroll
-    for (int d = 0; d < NDIM; ++d) x[d] = map_f64(X[d], d, N, sm, J, slot[d]);
+    for (int d = 0; d < NDIM; ++d) {
+        x[d] = map_f64(X[d], d, N, sm, J, slot[d]);
+        if (d % 8 == 7) J *= sm.n8;
+    }
+    if (NDIM % 8) J *= sm.nr;
     if constexpr (I::kMode == 1) {
         if (!EDGE || valid) store_point<NDIM, double>(A, (long long)(q * 32ull + (unsigned long long)lane - start), x);
         return;
@@ -837,22 +893,35 @@ __device__ __forceinline__ void sample_block(const SampleArgs<double> &A, const 
             double v = J * f;
             if (EDGE && !valid) v = 0.0;
             P.s1[c] += v;
-            P.s2[c] += v * v;
+            P.s2[c] = __fma_rn(v, v, P.s2[c]);
             if (c == 0) f0 = v;
         }
     }
-    if (!EDGE || valid) {
-        const double h = f0 * f0;
-        if (hmode == kHistWarpPlain) {
-            // the warp's own copy: its 32 points are in 32 distinct bins
+    // (an invalid point adds 0)
+    const double h = f0 * f0;
+    if (hmode == kHistWarpPhased) {
+        // the warp's own copy: the lanes of a phase are in distinct bins
+        // (one phase for N = 2^L >= 32)
+        const unsigned mask = (unsigned)(A.map.priv - 1) << 27;
+#pragma unroll 1
+        for (unsigned ph = 0; ph <= mask; ph += 1u << 27) {
+            // (a few axes' bins read first, then written, as in FP32)
 #pragma unroll
-            for (int d = 0; d < NDIM; ++d) sm.h[d * sm.hs + slot[d]] += h;
-        } else {
+            for (int d0 = 0; d0 < NDIM; d0 += kHistBatch) {
+                double hv[kHistBatch];
 #pragma unroll
-            for (int d = 0; d < NDIM; ++d) atomicAdd(&sm.h[d * sm.hs + slot[d]], h);
+                for (int d = d0; d < d0 + kHistBatch && d < NDIM; ++d)
+                    if (((unsigned)(X[d] >> 32) & mask) == ph) hv[d - d0] = sm.h[d * sm.stride + slot[d]];
+#pragma unroll
+                for (int d = d0; d < d0 + kHistBatch && d < NDIM; ++d)
+                    if (((unsigned)(X[d] >> 32) & mask) == ph) sm.h[d * sm.stride + slot[d]] = hv[d - d0] + h;
+            }
+            __syncwarp();
         }
+    } else {
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d) atomicAdd(&sm.h[d * sm.stride + slot[d]], h);
     }
-    if (hmode == kHistWarpPlain) __syncwarp();
 }
 
 // nsteps consecutive 32-point blocks starting at block q0, every lane's
@@ -997,10 +1066,9 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
     }
     const int N = I::nbins(A.nbins);
     const int ncomp = A.g.ncomp;
-    const bool priv = sizeof(Real) == 4 && POW2 && I::priv(A.map);
-    // FP64: warp copies for Sobol points and N = 2^L >= 32 when they fit
-    const bool priv64 = sizeof(Real) == 8 && I::kGen != 2 && A.map.priv != 0;
-    const int hmode = (priv || priv64) ? kHistWarpPlain : kHistBlock;
+    // warp copies of the histogram for Sobol points when they fit
+    const bool priv = I::kGen != 2 && (sizeof(Real) == 4 ? I::priv(A.map) : A.map.priv != 0);
+    const int hmode = !priv ? kHistBlock : (sizeof(Real) == 4 && POW2 ? kHistWarpPlain : kHistWarpPhased);
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem<Real> sm;
@@ -1024,18 +1092,18 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
             stage_grid_f32(sm.ew, NDIM, N, N, A.edges, A.map);
         }
     } else {
-        sm.stride = kStride;
+        sm.stride = N;
         sm.ew = reinterpret_cast<double2 *>(smem_raw);
-        double *hist = reinterpret_cast<double *>(sm.ew + NDIM * kStride);
-        // the block's histogram (kStride slots per axis), or every warp's [NDIM][N]
-        sm.hs = priv64 ? N : kStride;
-        sm.h = priv64 ? hist + (threadIdx.x >> 5) * NDIM * N : hist;
-        for (int i = threadIdx.x; i < (priv64 ? kWarpsPerBlock * NDIM * N : NDIM * kStride); i += blockDim.x)
-            hist[i] = 0.0;
+        sm.n8 = jacobian_scale(N, 8);
+        sm.nr = jacobian_scale(N, NDIM % 8);
+        double *hist = reinterpret_cast<double *>(sm.ew + NDIM * N);
+        // every warp's [NDIM][N], or the block's
+        sm.h = priv ? hist + (threadIdx.x >> 5) * NDIM * N : hist;
+        for (int i = threadIdx.x; i < (priv ? kWarpsPerBlock : 1) * NDIM * N; i += blockDim.x) hist[i] = 0.0;
         for (int idx = threadIdx.x; idx < NDIM * N; idx += blockDim.x) {
             const int d = idx / N, k = idx - d * N;
             const double *e = A.edges + (size_t)d * (N + 1);
-            sm.ew[d * kStride + k] = make_double2(e[k], e[k + 1] - e[k]);
+            sm.ew[idx] = make_double2(e[k], e[k + 1] - e[k]);
         }
     }
     __syncthreads();
@@ -1047,7 +1115,6 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
     const unsigned long long end = start + (unsigned long long)n;
     const unsigned long long qb = (end + 31ull) >> 5;
     const unsigned long long nblk = n > 0 ? qb - qa : 0ull;
-    const unsigned long long gwarp = (unsigned long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
     const unsigned long long twarps = (unsigned long long)gridDim.x * kWarpsPerBlock;
     unsigned long long plen = (nblk + twarps - 1) / twarps;
     if (plen < (unsigned long long)A.chunk_min) plen = A.chunk_min;
@@ -1055,8 +1122,15 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
     // time all warps read or write within one window of the point arrays
     // (DRAM locality) instead of one long stretch each
     if (I::kMode != 0 && plen > kRun) plen = kRun;
-    plen = (plen + 1ull) & ~1ull;
+    // (an FP64 pass may give a warp a single block)
+    if (sizeof(Real) == 4 || plen > 1) plen = (plen + 1ull) & ~1ull;
     const unsigned long long nchunk = (nblk + plen - 1) / plen;
+    // Chunks go to warps CTA by CTA; in a pass with chunks for at most half
+    // the warps, to warp 0 of every CTA, then warp 1, ..., so that every SM
+    // is loaded alike.  (A full pass is 1.2% slower that way.)
+    const unsigned long long gwarp = I::kMode == 0 && 2 * nchunk <= twarps
+        ? (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x
+        : (unsigned long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
 
     Acc<Real> s1[CV_MAX_COMP], s2[CV_MAX_COMP];
 
@@ -1121,14 +1195,14 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
             } else {
                 v = hist[d * N + p];
             }
-        } else if (priv64) {
+        } else if (priv) {
             // the warps' copies, summed in warp order
-            const double *hist = reinterpret_cast<const double *>(sm.ew + NDIM * kStride);
+            const double *hist = reinterpret_cast<const double *>(sm.ew + NDIM * N);
             v = 0.0;
 #pragma unroll
-            for (int w = 0; w < kWarpsPerBlock; ++w) v += hist[(w * NDIM + d) * N + k];
+            for (int w = 0; w < kWarpsPerBlock; ++w) v += hist[w * NDIM * N + idx];
         } else {
-            v = sm.h[d * kStride + k];
+            v = sm.h[idx];
         }
         if (parts) ph[d * N + k] = v;
         else if (v != Real(0)) atomicAdd(&A.H[d * N + k], (double)v);
@@ -1321,7 +1395,7 @@ k_batch_sample(const BatchSampleArgs B)
             const unsigned per = ((((unsigned)tile.nblk + kWarpsPerBlock - 1) / kWarpsPerBlock) + 1u) & ~1u;
             const unsigned long long w0 = tile.q0 + (unsigned long long)warp * per;
             const unsigned long long w1 = min(w0 + per, tile.q0 + (unsigned long long)tile.nblk);
-            const int hmode = A.map.priv ? kHistWarpPlain : kHistWarpAtomic;
+            constexpr int hmode = POW2 ? kHistWarpPlain : kHistWarpPhased;
             if (w0 < w1) {
                 unsigned X[NDIM];
                 sobol_skip<NDIM, unsigned>(X, w0, lane, POW2 ? A.map.li : 0);

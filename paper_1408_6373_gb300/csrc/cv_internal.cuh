@@ -129,7 +129,8 @@ struct MapParams {
     int li;                         // direction table: L - 4 (permuted words), else 0
     unsigned sA;                    // byte offset of the bin's grid entry = word >> sA, sA = 29 - L
     int G;                          // the fraction sits 2^-G below the mantissa's top (G = max(0, L - 6))
-    int priv;                       // per-warp f^2 histograms updated without atomics
+    int priv;                       // per-warp f^2 histograms updated without atomics, in this
+                                    // many steps (hist_phases); 0: shared-memory atomics
 };
 
 // The FP32 sampling kernels' table entry of a bin with left edge e and
@@ -394,19 +395,13 @@ void fill_genz_params(const cv_genz *g, GenzParams<Real> *p);
 int fp32_range_check(const cv_genz *g, char *msg, size_t len);
 #endif  // !__CUDACC_RTC__
 
-// Shared memory of a sampling block.  FP64: grid {e, w} with CV_MAX_BINS
-// slots per axis, then the block's histogram with CV_MAX_BINS slots per
-// axis or, with private histograms, one [ndim][nbins] copy per warp.  FP32: the grid table [ndim][nbins] (8-byte
-// entries, aligned to 8 nbins bytes), then either one block histogram
-// [ndim][nbins] of floats or, with private histograms, one such copy per
-// warp.
+// Shared memory of a sampling block: the grid table [ndim][nbins] (FP64:
+// 16-byte {e, w} entries; FP32: 8-byte entries, aligned to 8 nbins bytes),
+// then either one block histogram [ndim][nbins] or, with private
+// histograms, one such copy per warp.
 inline size_t sample_smem_bytes(int ndim, int nbins, bool fp64, bool priv) {
-    if (fp64)
-        return (size_t)ndim * CV_MAX_BINS * 2 * sizeof(double) +
-               (priv ? (size_t)kWarpsPerBlock * ndim * nbins : (size_t)ndim * CV_MAX_BINS) * sizeof(double);
-    return (size_t)ndim * nbins * 2 * sizeof(float) +
-           (priv ? (size_t)kWarpsPerBlock * ndim * nbins : (size_t)ndim * nbins) * sizeof(float) +
-           8 * (size_t)nbins;  // (to align the grid to 8 nbins bytes)
+    const size_t entries = (size_t)ndim * nbins * (2 + (priv ? kWarpsPerBlock : 1));
+    return fp64 ? entries * sizeof(double) : entries * sizeof(float) + 8 * (size_t)nbins;
 }
 
 // Resident 256-thread blocks per SM the FP32 sampling kernels are compiled
@@ -417,16 +412,31 @@ constexpr size_t kSmemPerSM = 228 * 1024;     // shared memory of one SM
 constexpr size_t kSmemBlockReserve = 2048;    // per block: runtime reserve + static arrays
 
 #if !defined(__CUDACC_RTC__)
+// Steps in which a warp updates its own f^2 histogram of N bins without
+// conflicts (at most 16).  The 32 Sobol points of an aligned block lie in 32
+// distinct 1/32-strata of every axis.  Powers of two: a bin is 32/N whole
+// strata (N < 32), so the lanes whose strata agree mod 32/N hit distinct
+// bins; from 32 bins on all lanes do.  Other N: two points m strata apart are
+// more than (m - 1)/32 apart, so for a power of two m with (m - 1)/32 >= 1/N
+// the lanes whose strata agree mod m hit distinct bins.  (An FP32 or FP64 add
+// on shared memory is a compare-and-swap loop on this GPU, and one copy for
+// the whole block makes the warps collide.)
+inline int hist_phases(int N)
+{
+    if ((N & (N - 1)) == 0) return N >= 32 ? 1 : 32 / N;
+    int m = 2;
+    while ((m - 1) * N < 32) m <<= 1;
+    return m;
+}
+
 // Map constants of an axis with N bins for the sampling kernels.
 //   N = 2^L >= 32: frac/N and the bin's slot come straight from the bits of
 //   the Sobol word (table li = L - 4 holds the words bit-permuted so that
 //   the slot is word >> (32 - L) and the fraction's bits sit at mantissa
 //   position: word & mF).  Other N take the generic map.
-//   priv: for N >= 32 the 32 points of an aligned block fall into 32
-//   distinct 1/32-strata of every axis, hence into 32 distinct bins, so a
-//   warp can keep its own f^2 histogram and update it with plain loads and
-//   stores.  Used on the FP32 path when every warp's copy fits beside the
-//   grid at the occupancy the kernel is compiled for.
+//   priv: a warp keeps its own f^2 histogram and updates it with plain loads
+//   and stores, in hist_phases(N) steps.  Used when every warp's copy fits beside
+//   the grid at the occupancy the kernel is compiled for.
 inline MapParams make_map(int N, int ndim, bool fp64)
 {
     MapParams m;
@@ -445,12 +455,12 @@ inline MapParams make_map(int N, int ndim, bool fp64)
         m.expE = (unsigned)(127 + m.G - L) << 23;
         m.li = L - 4;
         m.sA = 29 - L;
-        const int blocks = min_blocks_f32(ndim);
-        // (FP64: the kernel is compiled for one block per SM; its copies must
-        // still leave room for a second)
-        m.priv = fp64 ? 2 * (sample_smem_bytes(ndim, N, true, true) + kSmemBlockReserve) <= kSmemPerSM
-                      : (size_t)blocks * (sample_smem_bytes(ndim, N, false, true) + kSmemBlockReserve) <= kSmemPerSM;
     }
+    // (FP64: the kernel is compiled for one block per SM; its copies must
+    // still leave room for a second)
+    const int blocks = fp64 ? 2 : min_blocks_f32(ndim);
+    if ((size_t)blocks * (sample_smem_bytes(ndim, N, fp64, true) + kSmemBlockReserve) <= kSmemPerSM)
+        m.priv = hist_phases(N);
     return m;
 }
 

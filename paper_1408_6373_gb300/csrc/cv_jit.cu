@@ -128,7 +128,7 @@ std::string policy_source(const SampleArgs<float> &a, int ndim, bool pow2)
     s += "  __device__ __forceinline__ static constexpr int table(const MapParams&) { return " +
          std::to_string(pow2 ? a.map.li : 0) + "; }\n";
     s += "  __device__ __forceinline__ static constexpr bool priv(const MapParams&) { return " +
-         std::string(pow2 && a.map.priv ? "true" : "false") + "; }\n";
+         std::string(a.map.priv ? "true" : "false") + "; }\n";
     s += "  __device__ __forceinline__ static constexpr int nbins(int) { return " + std::to_string(a.nbins) +
          "; }\n";
     s += "};\n}\n";
@@ -221,7 +221,7 @@ int jit_sample_kernel(int device, const SampleArgs<float> &a, int ndim, bool pow
 {
     std::string key("S");
     const int v[8] = {device, ndim, pow2 ? 1 : 0, min_blocks, a.nbins, a.gen == kGenPseudo ? 1 : 0,
-                      pow2 ? a.map.li : 0, pow2 && a.map.priv ? 1 : 0};
+                      pow2 ? a.map.li : 0, a.map.priv ? 1 : 0};
     key_add(key, v, sizeof(v));
     key_add(key, &a.g, sizeof(a.g));  // (GenzParams is zeroed before it is filled)
     {
@@ -233,7 +233,7 @@ int jit_sample_kernel(int device, const SampleArgs<float> &a, int ndim, bool pow
         }
     }
     const int rc = jit_load(device, specialised_source(a, ndim, pow2, min_blocks), "cv_jit_sample",
-                            sample_smem_bytes(ndim, a.nbins, false, pow2 && a.map.priv), out, err);
+                            sample_smem_bytes(ndim, a.nbins, false, a.map.priv != 0), out, err);
     if (rc == 0) {
         std::lock_guard<std::mutex> lk(g_mu);
         g_fast[key] = *out;
