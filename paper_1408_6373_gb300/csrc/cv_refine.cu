@@ -12,8 +12,6 @@
 // chi^2 = sum_j (I_j - mean)^2 / var_j without cancellation; the chi-square
 // probability P((m-1)/2, chi^2/2) uses the regularized incomplete gamma
 // function (series for x < a+1, Legendre continued fraction otherwise).
-#include <cfloat>
-
 #include "cv_internal.cuh"
 
 namespace cv {
@@ -66,42 +64,188 @@ __device__ __forceinline__ void stage_axis(int d, int N, const double *edges, fl
         ew32[(size_t)d * N + slot_of_bin(k, map)] = grid_entry_f32(e[k], e[k + 1] - e[k], N, map);
 }
 
-__device__ __forceinline__ double warp_sum_d(double v)
+// ---- the refinement's arithmetic: 64-bit integers in place of FP64
+//
+// A dependent FP64 operation takes 65 to 130 cycles on this GPU (two FP64
+// lanes per SM serve all its warps), a reciprocal 430, a square root 670, a
+// logarithm 2000; the refinement of an axis was a chain of them, 14.3
+// thousand cycles for 128 bins.  64-bit integer multiplications are four
+// 32-bit ones in ~25 cycles, so the compression's logarithm, division and
+// 1.5th power, the sums and the rebinning run on 64-bit fixed-point values
+// and 64-bit mantissas with their own exponent: 5.6 thousand cycles.  Every
+// quantity carries at least 2^-55 of its scale (a sum 2^-54 of its largest
+// term), against 2^-53 per operation in FP64: against 113-bit arithmetic the
+// edges of 128 bins are off by at most 8e-17 (random histograms; the FP64
+// chain 1.1e-15) and 7e-16 (contents over 17 decades; 9e-15).  Prefix sums
+// of integers are exact, so an even histogram reproduces its grid exactly.
+
+// The special-function unit's 1/x and 1/sqrt(x), good to ~2^-22.
+__device__ __forceinline__ float rcp_seed(float x)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
-// Maximum of non-negative doubles through their bit patterns: for x, y >= 0
-// the IEEE order is the order of the 64-bit integers, and integer compares
-// avoid the long FP64 latency of this part.
-__device__ __forceinline__ long long warp_max_bits(long long v)
+__device__ __forceinline__ float rsqrt_seed(float x)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
-// Refine axis `d` of the grid in place (one CTA of at least N threads, at
-// most 256).  Every reduction has a fixed order, so the result is
-// reproducible.  GB300 issues FP64 at a small fraction of the FP32 rate, so
-// the CTA is sized to the bins (idle warps would still spend FP64 issue
-// slots on the reductions), the per-axis scalars (1/s, 1/max r, R/N) are
-// computed once, and the per-bin divisions other than the smoothing's are
-// multiplications by correctly rounded reciprocals (each result within
-// 1.5 ulp of the quotient).  FP64 results take ~200 cycles here, so the
-// refinement is bound by its chain of dependent FP64 operations: maxima
-// and searches over non-negative doubles compare bit patterns instead.
-// The G blocks' partial histograms of axis d, summed into sH[0, N) by all
-// the CTA's threads: thread t takes the V-wide column q = t mod (N/V) of
-// the rows r, r + R, r + 2R, ... (r = t div (N/V), R row groups), so a
-// warp's loads are contiguous vectors and each thread keeps four in flight;
-// the R group sums of a bin are then added in group order.  FP32 partials
-// are summed with Kahan's compensation in FP32 throughout (FP64 throughput,
-// conversions included, is a small fraction of FP32 here) and converted
-// once per bin; FP64 partials are summed in FP64.  The assignment of rows
-// to threads is fixed, so the same partials give the same bits.  Called by
-// every thread of the CTA (it synchronises).
+// A non-negative value m 2^e with the top bit of m set, or m = 0.
+struct Wide {
+    unsigned long long m;
+    int e;
+};
+
+__device__ __forceinline__ Wide normalised(unsigned long long m, int e)
+{
+    const int lz = m ? __clzll((long long)m) : 0;
+    return {m << lz, m ? e - lz : -100000};
+}
+
+// A finite double >= 0.
+__device__ __forceinline__ Wide wide_of(double v)
+{
+    const unsigned long long b = (unsigned long long)max(__double_as_longlong(v), 0ll);  // (-0 is 0)
+    const int e = (int)(b >> 52);
+    const unsigned long long f = b & 0xfffffffffffffull;
+    return normalised(e ? f | 0x10000000000000ull : f, (e ? e : 1) - 1075);
+}
+
+__device__ __forceinline__ unsigned long long shr64(unsigned long long v, int n)
+{
+    return n > 63 ? 0ull : v >> n;
+}
+
+// 2^126 / m for a mantissa m (top bit set), to about 2^-60 of it: the
+// special-function unit's reciprocal y, then y (1 + e + e^2) with the exact
+// residual e = 1 - m y (Newton's iteration and its next term).
+__device__ __forceinline__ unsigned long long wide_rcp(unsigned long long m)
+{
+    const float y = rcp_seed((float)(unsigned)(m >> 32));            // 2^-32 / (m 2^-64)
+    const unsigned Y = (unsigned)(y * 4611686018427387904.0f);       // 2^30 / (m 2^-64), <= 2^31
+    const long long E = (1ll << 62) - (long long)__umul64hi(m, (unsigned long long)Y << 32);
+    const long long q = E >> 16;
+    const long long C = E + ((q * q) >> 30);
+    return ((unsigned long long)Y << 32) +
+           (unsigned long long)(__mul64hi((long long)((unsigned long long)C << 22), (long long)Y << 31) >> 19);
+}
+
+// Logarithms base 2 by table and series (Tang 1990): for f in [1 + i/128, 1 +
+// (i+1)/128), c_i = ceil(2^22 / (128 + i)) 2^-15 makes f c_i = 1 + z with
+// 0 <= z < 2^-7 + 2^-15, exactly; t_i = -log2 c_i.
+struct LogTable {
+    unsigned long long t[128];  // 2^64 t_i
+    unsigned c[128];            // 2^15 c_i
+};
+constexpr LogTable make_log_table()
+{
+    LogTable T{};
+    for (int i = 0; i < 128; ++i) {
+        const unsigned c = ((1u << 22) + 127u + (unsigned)i) / (128u + (unsigned)i);
+        T.c[i] = c;
+        // the bits of log2 y, y = 2^15 / c in [1, 2), by repeated squaring
+        unsigned __int128 y = ((unsigned __int128)1 << (15 + 63)) / c;
+        unsigned long long l = 0;
+        for (int b = 63; b >= 0; --b) {
+            y = (y * y) >> 63;
+            if (y >> 64) {
+                l |= 1ull << b;
+                y >>= 1;
+            }
+        }
+        T.t[i] = l;
+    }
+    return T;
+}
+__device__ const LogTable g_log = make_log_table();
+
+// 2^64 log2 f for f = m 2^-63 in [1, 2).
+__device__ __forceinline__ unsigned long long wide_log2(unsigned long long m, const LogTable &T)
+{
+    const int i = (int)(m >> 56) & 127;
+    const unsigned c = T.c[i];
+    // m c - 2^78, in units of 2^-70 (the integer bit drops out mod 2^64)
+    const unsigned long long p0 = (unsigned long long)(unsigned)m * c;
+    const unsigned long long p1 = (m >> 32) * c + (p0 >> 32);
+    const unsigned long long z = (p1 << 24) + ((p0 & 0xffffffffull) >> 8);
+    // ln(1 + z) = z (1 - z (1/2 - z (1/3 - ...))), the terms from z^5 on in
+    // 32 bits
+    const unsigned zh = (unsigned)(z >> 32);
+    unsigned a = 613566757u - (__umulhi(zh, 536870912u) >> 6);       // 1/7 - z/8
+    a = 715827883u - (__umulhi(zh, a) >> 6);                         // 1/6 - z a
+    a = 858993459u - (__umulhi(zh, a) >> 6);                         // 1/5 - z a
+    unsigned long long A = 4611686018427387904ull - (__umul64hi(z, (unsigned long long)a << 32) >> 6);  // 1/4 - z a
+    A = 6148914691236517205ull - (__umul64hi(z, A) >> 6);            // 1/3 - z A
+    A = 9223372036854775808ull - (__umul64hi(z, A) >> 6);            // 1/2 - z A
+    const unsigned long long u = __umul64hi(z, A) >> 6;              // z A
+    const unsigned long long w = z - __umul64hi(z, u);               // 2^70 ln(1 + z)
+    return T.t[i] + (__umul64hi(w, 13306513097844322492ull) >> 5);   // log2 e, 2^63
+}
+
+// (y / -log2(1 - y))^1.5 for x = 1 - y = f 2^-k, f = m 2^-63 in [1, 2), k >= 1:
+// the compressed weight ((1 - x) / ln(1/x))^1.5 up to the constant factor
+// (ln 2)^1.5, in units of 2^-64.  x = 1 gives kCompressOne.
+constexpr unsigned long long kCompressOne = 10645300222249006184ull;  // (ln 2)^1.5 2^64
+__device__ __forceinline__ unsigned long long compress_weight(unsigned long long m, int k, const LogTable &T)
+{
+    const unsigned long long X = shr64(m, k - 1);  // x
+    Wide n = normalised(X ? 0ull - X : ~0ull, 0);  // y = n.m 2^(n.e - 64)
+    Wide D;                                        // -log2 x = D.m 2^(D.e - 64)
+    if (n.e > -6) {
+        const int b = 32 - __clz(k);               // k < 2^b
+        D = normalised(((unsigned long long)(unsigned)k << (64 - b)) - (wide_log2(m, T) >> b), b);
+    } else {
+        // x near 1, where the logarithm cancels: y log2 e (1 + y/2 + y^2/3 + ...)
+        const unsigned long long y = shr64(n.m, -n.e);
+        unsigned long long a = 1676976733973595601ull;               // 1/11
+        a = 1844674407370955161ull + __umul64hi(y, a);               // 1/10 + y a
+        a = 2049638230412172401ull + __umul64hi(y, a);
+        a = 2305843009213693952ull + __umul64hi(y, a);
+        a = 2635249153387078802ull + __umul64hi(y, a);
+        a = 3074457345618258602ull + __umul64hi(y, a);
+        a = 3689348814741910323ull + __umul64hi(y, a);
+        a = 4611686018427387904ull + __umul64hi(y, a);
+        a = 6148914691236517205ull + __umul64hi(y, a);
+        a = 9223372036854775808ull + __umul64hi(y, a);               // 1/2 + y/3 + ...
+        const unsigned long long l = 13306513097844322492ull;        // log2 e, 2^63
+        const unsigned long long s = l + __umul64hi(l, __umul64hi(y, a));  // < 2^64 (y < 2^-6)
+        D = normalised(__umul64hi(n.m, s), n.e + 1);
+    }
+    // q = y / D: sqrt q = y / sqrt(y D), with 1 / sqrt v from the
+    // special-function unit's w and w (1 + e/2 + 3/8 e^2), e = 1 - v w^2
+    unsigned long long v = __umul64hi(n.m, D.m);                     // [2^62, 2^64)
+    int ev = n.e + D.e;
+    if (ev & 1) {
+        v >>= 1;
+        ++ev;
+    }
+    const float wf = rsqrt_seed((float)(unsigned)(v >> 32));         // 2^-16 / sqrt(v 2^-64)
+    const unsigned W = (unsigned)(wf * 35184372088832.0f);           // 2^29 w, w < 2.83
+    const long long E = (1ll << 60) - (long long)__umul64hi(v, ((unsigned long long)W * W) << 2);
+    const long long h = E >> 16;
+    const long long C = (E >> 1) + ((3 * ((h * h) >> 28)) >> 3);
+    const unsigned long long w = ((unsigned long long)W << 33) +
+        (unsigned long long)(__mul64hi((long long)((unsigned long long)C << 23), (long long)W << 31) >> 17);  // 2^62 w
+    // sqrt q = n w 2^(n.e - ev/2) < 0.84
+    const int sh = ev / 2 - n.e - 2;
+    const unsigned long long r1 = __umul64hi(n.m, w);
+    const unsigned long long u = sh >= 0 ? shr64(r1, sh) : r1 << -sh;
+    return __umul64hi(__umul64hi(u, u), u);
+}
+
+// f 2^-64 as a double, rounded to nearest.
+__device__ __forceinline__ double unit_double(unsigned long long f)
+{
+    const int lz = __clzll((long long)f);
+    const unsigned long long m = f << (lz & 63);
+    const unsigned long long v = ((unsigned long long)(1021 - lz) << 52) + (((m >> 10) + 1ull) >> 1);
+    return __longlong_as_double((long long)(f ? v : 0ull));
+}
+
+// ---- sums of the passes' partial rows
 template <typename T, int V>
 __device__ __forceinline__ void load_vec(const T *p, T (&v)[V])
 {
@@ -119,232 +263,350 @@ __device__ __forceinline__ void load_vec(const T *p, T (&v)[V])
     }
 }
 
-// s + y with the running compensation c (Kahan), FP32
-__device__ __forceinline__ void kahan_add(float &s, float &c, float y)
-{
-    const float t = y - c;
-    const float u = s + t;
-    c = (u - s) - t;
-    s = u;
-}
-
-// Group sums: FP32 as (sum, compensation) pairs, FP64 as (sum, 0).
-template <typename T>
-struct GroupSum { using type = float2; };
-template <>
-struct GroupSum<double> { using type = double2; };
-
-template <typename T, int V>
-__device__ __forceinline__ void sum_rows(const T *P, int G, size_t nh, int N,
-                                         typename GroupSum<T>::type *grp)
-{
-    const int cols = N / V, R = (int)blockDim.x / cols;
-    const int t = threadIdx.x, q = t % cols, r = t / cols;
-    if (r >= R) return;
-    T s[V], c[V];
+// A running sum of V neighbouring values: FP32 with Kahan's compensation
+// (value s - c, kept as s and n = -c), two values per packed instruction;
+// FP64 plain.
+template <int V>
+struct Sum32 {
+    float s[V], n[V];
+    __device__ __forceinline__ void clear()
+    {
 #pragma unroll
-    for (int i = 0; i < V; ++i) s[i] = c[i] = T(0);
-    auto add = [&](const T (&v)[V]) {
+        for (int i = 0; i < V; ++i) s[i] = n[i] = 0.0f;
+    }
+    __device__ __forceinline__ void add(const float (&v)[V])
+    {
+        if constexpr (V == 1) {
+            const float y = v[0] + n[0];
+            const float u = s[0] + y;
+            n[0] = y - (u - s[0]);
+            s[0] = u;
+        } else {
+            const float2 m1 = make_float2(-1.0f, -1.0f);
+#pragma unroll
+            for (int i = 0; i < V; i += 2) {
+                const float2 s2 = make_float2(s[i], s[i + 1]);
+                const float2 y = __fadd2_rn(make_float2(v[i], v[i + 1]), make_float2(n[i], n[i + 1]));
+                const float2 u = __fadd2_rn(s2, y);
+                const float2 d = __ffma2_rn(s2, m1, u);
+                const float2 c = __ffma2_rn(d, m1, y);
+                s[i] = u.x;
+                s[i + 1] = u.y;
+                n[i] = c.x;
+                n[i + 1] = c.y;
+            }
+        }
+    }
+};
+// One value's sum in a group, (s, n) or the FP64 sum.
+__device__ __forceinline__ void group_add(float2 &a, const float2 &b)
+{
+    Sum32<1> t{{a.x}, {a.y}};
+    const float x[1] = {b.x}, y[1] = {b.y};
+    t.add(x);
+    t.add(y);
+    a = make_float2(t.s[0], t.n[0]);
+}
+__device__ __forceinline__ void group_add(double &a, const double &b) { a += b; }
+__device__ __forceinline__ float2 group_peer(const float2 &a, int o)
+{
+    return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+}
+__device__ __forceinline__ double group_peer(const double &a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ double group_value(const float2 &a) { return (double)a.x + (double)a.y; }
+__device__ __forceinline__ double group_value(const double &a) { return a; }
+
+template <int V>
+struct Sum64 {
+    double s[V];
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int i = 0; i < V; ++i) s[i] = 0.0;
+    }
+    __device__ __forceinline__ void add(const double (&v)[V])
+    {
+#pragma unroll
+        for (int i = 0; i < V; ++i) s[i] += v[i];
+    }
+};
+
+// Space of the row groups' sums of a CTA of 1024 threads, and of one of 256
+// (then the bins' prefix sums, weights and reciprocals).
+constexpr int kGroupBytes = 4352 * 8, kGroupBytesBatch = 1152 * 8;
+static_assert(kGroupBytesBatch >= (3 * CV_MAX_BINS + 1) * 8, "the bins' 64-bit values fit");
+
+// The sums over the G partial rows of one axis (first row P, row stride nh)
+// into sH, by all the CTA's threads: R groups of threads take every R-th
+// row, each thread a V-wide column, eight rows in flight (the rows come from
+// L2 at ~64 bytes a clock: 3.6 thousand cycles for 456 rows of 128 floats,
+// which four CTAs in a cluster would read in a quarter, for as many cycles
+// of cluster barriers and distributed reads); then every bin's R group sums
+// are added by T threads and a shuffle tree.  The order is fixed, so the
+// same rows give the same bits.  FP32 rows are summed with compensation in
+// FP32 (FP64 throughput is a small fraction of it here).  Called by every
+// thread of the CTA; synchronises before it returns.
+template <int GROUP, typename T, template <int> class S, typename E, int V>
+__device__ __forceinline__ void sum_rows(const CombineArgs *pa, int d, int N, unsigned char *raw, double *sH,
+                                         const MapParams *map)
+{
+    // (the sums first, converted by the bins' warps alone: an FP64
+    // instruction of each of 32 warps takes 512 cycles)
+    E *sums = reinterpret_cast<E *>(sH);
+    E *grp = reinterpret_cast<E *>(raw);
+    const int G = pa->part_G;
+    const size_t nh = (size_t)pa->part_nh;
+    // threads per bin, and a group stride that keeps their reads apart in
+    // the banks
+    const int lT = min(5, 31 - __clz((int)blockDim.x / N));
+    const int T2 = 1 << lT;
+    const int stride = ((N + 15) & ~15) + (lT >= 4 ? 1 : 16 >> lT);
+    const int cols = N / V;
+    int R = min(min((int)blockDim.x / cols, GROUP / (int)(sizeof(E) * stride)), G);
+    const int t = threadIdx.x, r = t / cols, q = t - r * cols;
+    if (r < R) {
+        S<V> s;
+        s.clear();
+        const T *p = static_cast<const T *>(pa->part_H) + (size_t)d * N + (size_t)q * V;
+        int b = r;
+        for (; b + 7 * R < G; b += 8 * R) {
+            T v[8][V];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) load_vec<T, V>(p + (size_t)(b + i * R) * nh, v[i]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) s.add(v[i]);
+        }
+        if (b + 3 * R < G) {
+            T v[4][V];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) load_vec<T, V>(p + (size_t)(b + i * R) * nh, v[i]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s.add(v[i]);
+            b += 4 * R;
+        }
+        if (b + R < G) {
+            T v[2][V];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) load_vec<T, V>(p + (size_t)(b + i * R) * nh, v[i]);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) s.add(v[i]);
+            b += 2 * R;
+        }
+        if (b < G) {
+            T v[V];
+            load_vec<T, V>(p + (size_t)b * nh, v);
+            s.add(v);
+        }
 #pragma unroll
         for (int i = 0; i < V; ++i) {
-            if constexpr (sizeof(T) == 4) kahan_add(s[i], c[i], v[i]);
-            else s[i] += v[i];
+            if constexpr (sizeof(T) == 4) grp[r * stride + q * V + i] = make_float2(s.s[i], s.n[i]);
+            else grp[r * stride + q * V + i] = s.s[i];
         }
-    };
-    const T *p = P + (size_t)q * V;
-    int b = r;
-    // (eight rows in flight, then four: the loads' latency, not their
-    // bandwidth, bounds this loop)
-    for (; b + 7 * R < G; b += 8 * R) {
-        T v[8][V];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) load_vec<T, V>(p + (size_t)(b + i * R) * nh, v[i]);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) add(v[i]);
     }
-    for (; b + 3 * R < G; b += 4 * R) {
-        T v0[V], v1[V], v2[V], v3[V];
-        load_vec<T, V>(p + (size_t)b * nh, v0);
-        load_vec<T, V>(p + (size_t)(b + R) * nh, v1);
-        load_vec<T, V>(p + (size_t)(b + 2 * R) * nh, v2);
-        load_vec<T, V>(p + (size_t)(b + 3 * R) * nh, v3);
-        add(v0);
-        add(v1);
-        add(v2);
-        add(v3);
+    __syncthreads();
+    const int k = t >> lT, j = t & (T2 - 1);
+    E s{};
+    if (k < N) {
+        int g = j;
+        if (g < R) s = grp[g * stride + k];
+        for (g += T2; g < R; g += T2) group_add(s, grp[g * stride + k]);
     }
-    for (; b < G; b += R) {
-        T v[V];
-        load_vec<T, V>(p + (size_t)b * nh, v);
-        add(v);
+    for (int o = 1; o < T2; o <<= 1) {
+        // (both peers add the lower lane's sum first)
+        const E other = group_peer(s, o);
+        E a = (j & o) ? other : s;
+        group_add(a, (j & o) ? s : other);
+        s = a;
     }
-#pragma unroll
-    for (int i = 0; i < V; ++i) grp[r * N + q * V + i] = {s[i], c[i]};
-}
-
-__device__ void sum_parts_axis(const CombineArgs *pa, int d, int N, double *sH, const MapParams *map)
-{
-    // R x N group sums, R N <= 4 blockDim (FP32), 2 blockDim (FP64)
-    __shared__ __align__(16) unsigned char grp_raw[4096 * sizeof(float2)];
-    const size_t nh = (size_t)pa->part_nh;
-    const int G = pa->part_G;
-    const int k = threadIdx.x;
-    if (pa->part_f32) {
-        float2 *grp = reinterpret_cast<float2 *>(grp_raw);
-        const float *P = static_cast<const float *>(pa->part_H) + (size_t)d * N;
-        const int V = N % 4 == 0 ? 4 : N % 2 == 0 ? 2 : 1;
-        if (V == 4) sum_rows<float, 4>(P, G, nh, N, grp);
-        else if (V == 2) sum_rows<float, 2>(P, G, nh, N, grp);
-        else sum_rows<float, 1>(P, G, nh, N, grp);
+    // (rows in slot order: the writer's stores are then contiguous, and one
+    // permuted store here costs nothing)
+    if (k < N && j == 0) sums[sizeof(T) == 4 && pa->part_slots ? bin_of_slot(k, *map) : k] = s;
+    __syncthreads();
+    if constexpr (sizeof(T) == 4) {
+        // (each thread its own slot)
+        if (t < N) sH[t] = group_value(sums[t]);
         __syncthreads();
-        if (k < N) {
-            const int R = (int)blockDim.x / (N / V);
-            float s = 0.0f, c = 0.0f;
-            for (int r = 0; r < R; ++r) {
-                const float2 g = grp[r * N + k];
-                kahan_add(s, c, g.x);
-                kahan_add(s, c, -g.y);
-            }
-            // (rows in slot order: the writer's stores are then contiguous,
-            // and one permuted store here costs nothing)
-            sH[pa->part_slots ? bin_of_slot(k, *map) : k] = (double)s - (double)c;
-        }
-    } else {
-        double2 *grp = reinterpret_cast<double2 *>(grp_raw);
-        const double *P = static_cast<const double *>(pa->part_H) + (size_t)d * N;
-        const int V = N % 2 == 0 ? 2 : 1;
-        if (V == 2) sum_rows<double, 2>(P, G, nh, N, grp);
-        else sum_rows<double, 1>(P, G, nh, N, grp);
-        __syncthreads();
-        if (k < N) {
-            const int R = (int)blockDim.x / (N / V);
-            double a[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int r = 0; r < R; ++r) a[r & 3] += grp[r * N + k].x;
-            sH[k] = (a[0] + a[1]) + (a[2] + a[3]);
-        }
     }
 }
 
-__device__ void refine_axis(int d, int N, double *H, double *edges, int zero_hist, float2 *ew32 = nullptr,
-                            const MapParams *map = nullptr, const CombineArgs *pa = nullptr)
+// Refine axis `d` of the grid in place, one CTA of at least N threads, all
+// of which call this.  `active`: nothing is written when it is 0 (waited for
+// only before the first write).
+template <int GROUP>
+__device__ void refine_axis(int d, int N, double *H, double *edges, int zero_hist, float2 *ew32,
+                            const MapParams *map, const CombineArgs *pa, const int *active)
 {
     double *Hd = H ? H + (size_t)d * N : nullptr;
     double *e = edges + (size_t)d * (N + 1);
-    __shared__ double sH[CV_MAX_BINS], sq[CV_MAX_BINS];
-    __shared__ double sC[CV_MAX_BINS + 1], se[CV_MAX_BINS + 1];
-    __shared__ double wred[32];
-    __shared__ double s_sum, s_inv, s_rmax, s_RN;
+    __shared__ __align__(16) unsigned char grp_raw[GROUP];
+    __shared__ LogTable s_log;
+    __shared__ double sH[CV_MAX_BINS], se[CV_MAX_BINS + 1], sdw[CV_MAX_BINS];
+    unsigned long long *sC = reinterpret_cast<unsigned long long *>(grp_raw);  // (after the row sums)
+    unsigned long long *sR = sC + CV_MAX_BINS + 1, *sI = sR + CV_MAX_BINS;
+    __shared__ unsigned long long wm[8], wt[8];
+    __shared__ int we[8];
     const int k = threadIdx.x;            // bin of this thread
     const int lane = k & 31, warp = k >> 5;
-    // the warps holding bins; the others (a CTA sized for the partial sums)
-    // only meet the barriers: the FP64 pipe is a small fraction of FP32 here
-    const int nw = (N + 31) >> 5;
-    const bool act = warp < nw;
-    const double invN = __drcp_rn((double)N);  // (off the dependent chain)
-
-    if (pa && pa->part_H) sum_parts_axis(pa, d, N, sH, map);
-    else if (k < N) sH[k] = Hd[k];
-    for (int i = k; i <= N; i += blockDim.x) se[i] = e[i];
-    __syncthreads();
-    const bool bad = k < N && !isfinite(sH[k]);
-    const bool nz = k < N && sH[k] != 0.0;
-    const int any_bad = __syncthreads_or(bad);
-    const int any_nz = __syncthreads_or(nz);
-    if (!any_bad && any_nz) {
-        // smoothing over the neighbours (correctly rounded: an even
-        // histogram stays exactly even)
-        double h = 0.0;
-        if (k < N) {
-            if (k == 0) h = __dmul_rn(__dadd_rn(sH[0], sH[1]), 0.5);
-            else if (k == N - 1) h = __dmul_rn(__dadd_rn(sH[N - 2], sH[N - 1]), 0.5);
-            else h = __ddiv_rn(__dadd_rn(__dadd_rn(sH[k - 1], sH[k]), sH[k + 1]), 3.0);
-        }
-        // s = sum_k h_k (warp sums, then the warps in order by one thread;
-        // the per-axis scalars are computed once and shared)
-        if (act) {
-            const double ws = warp_sum_d(h);
-            if (lane == 0) wred[warp] = ws;
-        }
-        __syncthreads();
-        if (k == 0) {
-            double t = 0.0;
-            for (int w = 0; w < nw; ++w) t = __dadd_rn(t, wred[w]);
-            s_sum = t;
-            s_inv = __drcp_rn(t);
-        }
-        __syncthreads();
-        const double s = s_sum;
-        // compression r = ((1 - h/s) / ln(s/h))^1.5 = ((x - 1) / ln x)^1.5,
-        // x = h/s in (0, 1]
-        double r = 0.0;
-        if (k < N && h != 0.0) {
-            const double x = __dmul_rn(h, s_inv);
-            if (h == s || !(x < 1.0)) {
-                r = 1.0;
-            } else {
-                const double q = __dmul_rn(__dadd_rn(x, -1.0), __drcp_rn(log(x)));
-                r = __dmul_rn(q, sqrt(q));
-            }
-        }
-        if (act) {
-            const long long wm = warp_max_bits(__double_as_longlong(r));
-            if (lane == 0) wred[warp] = __longlong_as_double(wm);
-        }
-        __syncthreads();
-        if (k == 0) {
-            long long t = 0;
-            for (int w = 0; w < nw; ++w) t = max(t, __double_as_longlong(wred[w]));
-            s_rmax = __longlong_as_double(t);
-            s_inv = t > 0 ? __drcp_rn(__longlong_as_double(t)) : 0.0;
-        }
-        __syncthreads();
-        const long long rmax_bits = __double_as_longlong(s_rmax);
-        if (rmax_bits > 0) {
-            // scale to max 1 (the largest bins exactly 1)
-            double c = 0.0;
-            if (act) {
-                r = (__double_as_longlong(r) == rmax_bits) ? 1.0 : __dmul_rn(r, s_inv);
-                if (k < N) sq[k] = r > 0.0 ? __drcp_rn(r) : 0.0;
-                // inclusive prefix sum C_(k+1) = r_0 + ... + r_k
-                c = r;
+    const int nw = (N + 31) >> 5;         // the warps holding bins
+    // (all loads first: they arrive while the rows are summed)
+    const int on = active ? *(const volatile int *)active : 1;
+    double e0 = 0.0, e1 = 0.0;
+    if (k < N) {
+        e0 = e[k];
+        e1 = e[k + 1];
+    }
+    unsigned long long lt[2];
+    unsigned lc[2];
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const double t = __shfl_up_sync(0xffffffffu, c, o);
-                    if (lane >= o) c = __dadd_rn(t, c);
-                }
-                if (lane == 31) wred[warp] = c;
+    for (int i = 0; i < 2; ++i) {  // (at least 64 threads)
+        const int at = k + i * (int)blockDim.x;
+        if (at < 128) {
+            lt[i] = g_log.t[at];
+            lc[i] = g_log.c[at];
+        }
+    }
+    if (pa && pa->part_H) {
+        if (pa->part_f32) {
+            if (N % 4 == 0) sum_rows<GROUP, float, Sum32, float2, 4>(pa, d, N, grp_raw, sH, map);
+            else if (N % 2 == 0) sum_rows<GROUP, float, Sum32, float2, 2>(pa, d, N, grp_raw, sH, map);
+            else sum_rows<GROUP, float, Sum32, float2, 1>(pa, d, N, grp_raw, sH, map);
+        } else {
+            if (N % 2 == 0) sum_rows<GROUP, double, Sum64, double, 2>(pa, d, N, grp_raw, sH, map);
+            else sum_rows<GROUP, double, Sum64, double, 1>(pa, d, N, grp_raw, sH, map);
+        }
+    } else {
+        if (k < N) sH[k] = Hd[k];
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int at = k + i * (int)blockDim.x;
+        if (at < 128) {
+            s_log.t[at] = lt[i];
+            s_log.c[at] = lc[i];
+        }
+    }
+    // (whole warps leave: the barriers below count the others)
+    if (!on || warp >= max(nw, 4)) return;
+    // 2^64 / N, at most N too small, from one 32-bit division
+    const unsigned q32 = 0xffffffffu / (unsigned)N;
+    const unsigned long long invN = ((unsigned long long)q32 << 32) + (unsigned long long)(0u - q32 * (unsigned)N) * q32;
+    if (k < N) {
+        se[k] = e0;
+        sdw[k] = e1 - e0;
+        if (k == N - 1) se[N] = e1;
+    }
+    const double hk = k < N ? sH[k] : 0.0;
+    const int any_bad = __syncthreads_or(k < N && !isfinite(hk));
+    const int any_nz = __syncthreads_or(hk != 0.0);
+    const bool act = warp < nw;  // (the other warps only meet the barriers)
+    if (!any_bad && any_nz) {
+        // smoothing over the neighbours, six times the mean: 2 (a + b + c)
+        // inside, 3 (a + b) at the ends (an even histogram stays exactly even)
+        Wide h{0, -100000};
+        if (k < N) {
+            const Wide b = wide_of(hk);
+            const Wide a = k > 0 ? wide_of(sH[k - 1]) : Wide{0, -100000};
+            const Wide c = k < N - 1 ? wide_of(sH[k + 1]) : Wide{0, -100000};
+            const int E = max(b.e, max(a.e, c.e));
+            const unsigned long long v = shr64(a.m, 4 + E - a.e) + shr64(b.m, 4 + E - b.e) + shr64(c.m, 4 + E - c.e);
+            h = normalised((k > 0 && k < N - 1 ? 2ull : 3ull) * v, E);
+        }
+        // s = sum_k h_k: every warp at its own largest exponent, then the
+        // warps at the largest of theirs
+        const int up = 32 - __clz(N);  // (N 2^(64 - up) <= 2^64)
+        if (act) {
+            const int E = __reduce_max_sync(0xffffffffu, h.e);
+            const unsigned long long f = (shr64(h.m, up - 1 + E - h.e) + 1ull) >> 1;
+            const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)f & 0x3fffffu);
+            const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(f >> 22) & 0x3fffffu);
+            const unsigned l2 = __reduce_add_sync(0xffffffffu, (unsigned)(f >> 44));
+            if (lane == 0) {
+                wm[warp] = (unsigned long long)l0 + ((unsigned long long)l1 << 22) + ((unsigned long long)l2 << 44);
+                we[warp] = E;
             }
-            __syncthreads();
-            if (act) {
-                double off = 0.0;
-                for (int w = 0; w < warp; ++w) off = __dadd_rn(off, wred[w]);
-                c = __dadd_rn(off, c);
-                if (k < N) sC[k + 1] = c;
-                if (k == 0) sC[0] = 0.0;
-                if (k == N - 1) s_RN = __dmul_rn(c, invN);  // R / N, R = C_N
+        }
+        __syncthreads();
+        // compression r = ((1 - x) / ln(1/x))^1.5, x = h/s in (0, 1], up to a
+        // constant factor
+        unsigned long long R = 0;
+        if (act) {
+            int E = we[0];
+            for (int w = 1; w < nw; ++w) E = max(E, we[w]);
+            unsigned long long t = 0;
+            for (int w = 0; w < nw; ++w) t += shr64(wm[w], E - we[w]);
+            const Wide s = normalised(t, E + up);
+            if (h.m) {
+                // x = h/s = f 2^-k, f in [1, 2)
+                const unsigned long long x = __umul64hi(h.m, wide_rcp(s.m));
+                const int lz = __clzll((long long)x);
+                const int ke = lz - 1 - h.e + s.e;
+                const unsigned long long r = ke <= 0 ? kCompressOne : compress_weight(x << lz, ke, s_log);
+                // (256 of them stay below 2^63)
+                R = ((r >> 8) + 1ull) >> 1;
             }
-            __syncthreads();
-            const int m = k;
-            if (m >= 1 && m < N) {
-                // new edge m at compressed weight t = m R / N
-                const double t = __dmul_rn((double)m, s_RN);
-                // largest j in [0, N-1] with C_j <= t (C, t >= 0: bit-pattern compares)
-                const long long tb = __double_as_longlong(t);
-                int lo = 0, hi = N - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (__double_as_longlong(sC[mid]) <= tb) lo = mid;
-                    else hi = mid - 1;
-                }
-                e[m] = __fma_rn(__dadd_rn(se[lo + 1], -se[lo]),
-                                __dmul_rn(__dadd_rn(t, -sC[lo]), sq[lo]), se[lo]);
+            // inclusive prefix sum C_(k+1) = r_0 + ... + r_k
+            unsigned long long c = R;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long p = __shfl_up_sync(0xffffffffu, c, o);
+                if (lane >= o) c += p;
             }
+            if (lane == 31) wt[warp] = c;
+            if (k < N) {
+                sR[k] = R;
+                // (its reciprocal, for the bins the new edges fall into)
+                const int lr = R ? __clzll((long long)R) : 0;
+                sI[k] = R ? wide_rcp(R << lr) : 0ull;
+                sC[k + 1] = c;
+                if (k == 0) sC[0] = 0ull;
+            }
+        }
+        __syncthreads();
+        // sC holds prefix sums within each warp's bins: the warps before add
+        // their totals
+        unsigned long long before = 0, total = 0;
+        for (int w = 0; w < nw; ++w) {
+            if (w < warp) before += wt[w];
+            total += wt[w];
+        }
+        if (k < N) sC[k + 1] += before;
+        __syncthreads();
+        if (k >= 1 && k < N && total) {
+            // new edge m = k at compressed weight t = m total / N, with total =
+            // qn N + rem (values below 2^16 are divided by N through a
+            // product with ceil(2^32 / N))
+            unsigned long long qn = __umul64hi(total, invN);
+            unsigned rem = (unsigned)(total - qn * (unsigned)N);
+            const unsigned more = __umulhi(rem, q32 + 1u);
+            qn += more;
+            rem -= more * (unsigned)N;
+            const unsigned long long t = (unsigned long long)k * qn + __umulhi((unsigned)k * rem, q32 + 1u);
+            // largest j in [0, N-1] with C_j <= t (then C_(j+1) > t, since t <
+            // C_N), by quarters: the three probes of a step load together
+            int lo = 0, len = N;  // the answer is in [lo, lo + len)
+            while (len > 1) {
+                const int h = (len + 3) >> 2;
+                const int p1 = min(lo + h, N), p2 = min(lo + 2 * h, N), p3 = min(lo + 3 * h, N);
+                const bool b1 = sC[p1] <= t, b2 = sC[p2] <= t, b3 = sC[p3] <= t;
+                lo += b3 ? 3 * h : b2 ? 2 * h : b1 ? h : 0;
+                len = h;
+            }
+            const unsigned long long r = sR[lo];
+            const int lr = r ? __clzll((long long)r) : 0;
+            const unsigned long long f = __umul64hi((t - sC[lo]) << lr, sI[lo]) << 2;
+            e0 = __fma_rn(sdw[lo], unit_double(f), se[lo]);
+            e[k] = e0;
         }
     }
     if (zero_hist && k < N) Hd[k] = 0.0;
     if (ew32) {
-        __syncthreads();  // (the new edges of this axis, written by every thread)
-        stage_axis(d, N, edges, ew32, *map, k, blockDim.x);
+        // the FP32 table of the new grid (as stage_axis)
+        __syncthreads();
+        if (k < N) se[k] = e0;
+        __syncthreads();
+        if (k < N)
+            ew32[(size_t)d * N + slot_of_bin(k, *map)] = grid_entry_f32(e0, se[k + 1] - e0, N, *map);
     }
 }
 
@@ -385,56 +647,84 @@ __global__ void __launch_bounds__(256) k_add_parts(const void *part_H, int G, in
 
 __global__ void __launch_bounds__(256) k_refine(int N, double *H, double *edges)
 {
-    refine_axis(blockIdx.x, N, H, edges, 0);
+    refine_axis<kGroupBytesBatch>(blockIdx.x, N, H, edges, 0, nullptr, nullptr, nullptr, nullptr);
 }
 
-// Per component: fold the iteration result into the combination; thread 0
+// Per component: fold the iteration result into the combination; lane 0
 // then updates the iteration control.  The chi-square probability is only
-// needed for the final answer and is evaluated when the run stops.
-__device__ void combine_iteration(const CombineArgs &A)
+// needed for the final answer and is evaluated when the run stops.  One CTA;
+// its first warp combines.
+__device__ void combine_iteration(const CombineArgs &A, const int *active)
 {
     DevState *st = A.st;
-    const int c = threadIdx.x;
-    const long long n = st->n_cur;
-    const int j = st->iter;
-    __shared__ int s_ok[CV_MAX_COMP];
-    __shared__ int s_bad[CV_MAX_COMP];
-    __shared__ int s_stop;
+    const int c = threadIdx.x, lane = c & 31, nwarp = (int)(blockDim.x >> 5);
+    const int on = active ? *(const volatile int *)active : 1;
+    __shared__ double wsum[32][2 * CV_MAX_COMP + 1];
     __shared__ double s_sum[2 * CV_MAX_COMP];
+    // every input first (independent loads)
+    const long long n = st->n_cur, neval0 = st->neval;
+    const int j = st->iter;
+    double sumI0 = 0.0, W0 = 0.0, mean0 = 0.0, M20 = 0.0;
+    int zero = 0;
+    if (c < A.ncomp) {
+        sumI0 = st->sumI[c];
+        W0 = st->W[c];
+        mean0 = st->mean[c];
+        M20 = st->M2[c];
+        zero = st->zero[c];
+    }
+    // FP64 latency is high, so divisions are reciprocal multiplications
+    // except where a reciprocal itself is the result; these two need no sum
+    const double inv_n = __drcp_rn((double)n);
+    const double inv_n1 = __drcp_rn((double)(n - 1));
     if (A.part_S) {
-        // the pass's sums, block partials added in block order: warp w takes
-        // values w, w + warps, ...; lane l the blocks l, l + 32, ..., then a
-        // fixed shuffle tree (as a pass's last block would)
-        const int lane = c & 31, nwarp = (int)(blockDim.x >> 5);
-        for (int v = c >> 5; v < 2 * A.ncomp; v += nwarp) {
-            double acc = 0.0;
-            for (int b = lane; b < A.part_G; b += 32) acc += __ldcg(&A.part_S[b * (2 * CV_MAX_COMP) + v]);
+        // The pass's sums, block partials added in a fixed order: thread i
+        // takes value i mod 2 ncomp of every so-many-th row, then the lanes
+        // and warps are added per value.  (Only the values in use: 32 lanes'
+        // additions cost 16 cycles of the SM's FP64 lanes.)
+        const int nv = 2 * A.ncomp, rows = 32 / nv, row = lane / nv, v = lane - row * nv;
+        double acc = 0.0;
+        if (row < rows) {
+            const int step = rows * nwarp;
+            int b = (c >> 5) * rows + row;
+            for (; b + 3 * step < A.part_G; b += 4 * step) {
+                double x[4];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) s_sum[v] = acc;
+                for (int i = 0; i < 4; ++i) x[i] = __ldcg(&A.part_S[(size_t)(b + i * step) * (2 * CV_MAX_COMP) + v]);
+                acc += (x[0] + x[1]) + (x[2] + x[3]);
+            }
+            for (; b < A.part_G; b += step) acc += __ldcg(&A.part_S[(size_t)b * (2 * CV_MAX_COMP) + v]);
+        }
+        // (row r of the warp's rows is at lanes r nv .. r nv + nv - 1)
+        for (int r = rows; r > 1; r = (r + 1) >> 1) {
+            const int h = (r + 1) >> 1;
+            const double o = __shfl_down_sync(0xffffffffu, acc, h * nv);
+            if (row + h < r) acc += o;
+        }
+        if (lane < nv) wsum[c >> 5][lane] = acc;
+        __syncthreads();
+        for (int w = c >> 5; w < nv; w += nwarp) {
+            double t = lane < nwarp ? wsum[lane][w] : 0.0;
+            for (int o = 16; o > 0; o >>= 1)
+                if (o < nwarp) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) s_sum[w] = t;
         }
         __syncthreads();
     }
+    if (!on || c >= 32) return;  // (one warp from here on)
+    bool ok = true, bad = false;
+    double chi2 = 0.0;
     if (c < A.ncomp) {
-        // every input first (independent loads), then the arithmetic: FP64
-        // latency is high, so divisions are reciprocal multiplications
-        // except where a reciprocal itself is the result
         const double S1 = A.part_S ? s_sum[2 * c] : st->S1[c];
         const double S2 = A.part_S ? s_sum[2 * c + 1] : st->S2[c];
-        const double sumI0 = st->sumI[c], W0 = st->W[c], mean0 = st->mean[c], M20 = st->M2[c];
-        int zero = st->zero[c];
-        const double dn = (double)n;
-        const double inv_n = __drcp_rn(dn);
-        const double inv_n1 = __drcp_rn((double)(n - 1));
         const double I = __dmul_rn(S1, inv_n);
         const double var = __dmul_rn(__fma_rn(-I, I, __dmul_rn(S2, inv_n)), inv_n1);
         if (A.log_I && j < A.log_cap) {
             A.log_I[j * CV_MAX_COMP + c] = I;
             A.log_var[j * CV_MAX_COMP + c] = var;
         }
-        const bool bad = !isfinite(I) || !isfinite(var);
+        bad = !isfinite(I) || !isfinite(var);
         if (bad) atomicOr(&st->status, 1);
-        s_bad[c] = bad;
         const int m = j + 1;
         const double sumI = sumI0 + I;
         st->sumI[c] = sumI;
@@ -452,10 +742,10 @@ __device__ void combine_iteration(const CombineArgs &A)
         } else {
             st->zero[c] = 1;
         }
-        double integral, error, chi2;
+        double integral, error;
         if (zero) {
             integral = sumI / (double)m;
-            error = chi2 = 0.0;
+            error = 0.0;
         } else {
             integral = mean;
             error = rsqrt(W);
@@ -465,83 +755,70 @@ __device__ void combine_iteration(const CombineArgs &A)
         st->error[c] = error;
         st->chi2[c] = chi2;
         const double tol = fmax(A.epsabs, A.epsrel * fabs(integral));
-        s_ok[c] = !bad && error <= tol;
+        ok = !bad && error <= tol;
         st->S1[c] = 0.0;
         st->S2[c] = 0.0;
     }
-    __syncthreads();
+    ok = __all_sync(0xffffffffu, ok);
+    bad = __any_sync(0xffffffffu, bad);
+    const long long neval = neval0 + n;
+    const long long next = A.nstart + (long long)(j + 1) * A.nincrease;
+    // (a non-finite iteration result -- the integrand returned NaN or Inf, or
+    // its squares overflowed -- stops the run unconverged)
+    const bool done = !bad && neval >= A.mineval && ok;
+    const bool stop = bad || done || neval + next > A.maxeval;
     if (c == 0) {
-        int ok = 1, bad = 0;
-        for (int i = 0; i < A.ncomp; ++i) {
-            ok &= s_ok[i];
-            bad |= s_bad[i];
-        }
-        const long long neval = st->neval + n;
         st->neval = neval;
         st->iter = j + 1;
-        const long long next = A.nstart + (long long)(j + 1) * A.nincrease;
-        int stop = 0;
-        if (bad) {
-            // a non-finite iteration result (the integrand returned NaN or
-            // Inf, or its squares overflowed): the run stops unconverged
-            st->fail = 1;
-            stop = 1;
-        } else if (neval >= A.mineval && ok) {
-            st->fail = 0;
-            stop = 1;
-        } else if (neval + next > A.maxeval) {
-            st->fail = 1;
-            stop = 1;
+        if (stop) {
+            st->fail = done ? 0 : 1;
         } else {
             st->next_index += (unsigned long long)n;
             st->n_cur = next;
         }
-        s_stop = stop;
     }
-    __syncthreads();
     if (c < A.ncomp) {
         const int m = j + 1;
-        st->prob[c] = (s_stop && !st->zero[c] && m > 1) ? gamma_p(0.5 * (m - 1), 0.5 * st->chi2[c]) : 0.0;
+        st->prob[c] = (stop && !zero && m > 1) ? gamma_p(0.5 * (m - 1), 0.5 * chi2) : 0.0;
     }
-    __syncthreads();
+    __syncwarp();
     // read by the next sampling launch only, so no block of this launch
     // sees the change
-    if (c == 0 && s_stop) st->stopped = 1;
-    if (c == 0 && A.host_stop) *(volatile int *)A.host_stop = s_stop;
+    if (c == 0 && stop) st->stopped = 1;
+    if (c == 0 && A.host_stop) *(volatile int *)A.host_stop = stop ? 1 : 0;
 }
 
 // One Vegas iteration after its sampling pass: blocks 0..ndim-1 refine one
 // axis each from the histogram (and clear it), block ndim combines the
-// iteration.  Runs only if the sampling launch before it ran.
+// iteration.  Writes nothing unless the sampling launch before it ran.
 __global__ void __launch_bounds__(1024)
 k_refine_combine(int ndim, int N, double *H, double *edges, const CombineArgs A, float2 *ew32, MapParams map)
 {
-    if (!*(volatile const int *)&A.st->pass_active) return;
-    if ((int)blockIdx.x < ndim) refine_axis(blockIdx.x, N, H, edges, 1, ew32, &map, &A);
-    else combine_iteration(A);
+    const int d = (int)blockIdx.x;
+    if (d < ndim) refine_axis<kGroupBytes>(d, N, H, edges, 1, ew32, &map, &A, &A.st->pass_active);
+    else combine_iteration(A, &A.st->pass_active);
 }
 
 // Start of a run: uniform grid e_k = k/N, empty histogram and sums, Sobol
-// index 1 (index 0, the all-zero point, is skipped).
-__global__ void k_reset(DevState *st, double *edges, double *H, int ndim, int N, long long nstart, float2 *ew32,
-                        MapParams map)
+// index 1 (index 0, the all-zero point, is skipped).  One CTA per axis: a
+// thread's one division, not ndim (N + 1) / threads of them in turn (54 us
+// for 30 axes of 256 bins in one CTA, 4 us so).
+__global__ void k_reset(DevState *st, double *edges, double *H, int N, long long nstart, float2 *ew32, MapParams map)
 {
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int stride = gridDim.x * blockDim.x;
-    for (int i = tid; i < ndim * (N + 1); i += stride) {
-        const int k = i % (N + 1);
-        edges[i] = (double)k / (double)N;
+    const int d = blockIdx.x;
+    double *e = edges + (size_t)d * (N + 1);
+    for (int k = threadIdx.x; k <= N; k += blockDim.x) e[k] = (double)k / (double)N;
+    for (int k = threadIdx.x; k < N; k += blockDim.x) H[(size_t)d * N + k] = 0.0;
+    if (d == 0) {
+        int *w = reinterpret_cast<int *>(st);
+        for (int i = threadIdx.x; i < (int)(sizeof(DevState) / sizeof(int)); i += blockDim.x) w[i] = 0;
     }
-    for (int i = tid; i < ndim * N; i += stride) H[i] = 0.0;
-    int *w = reinterpret_cast<int *>(st);
-    for (int i = tid; i < (int)(sizeof(DevState) / sizeof(int)); i += stride) w[i] = 0;
     __syncthreads();
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (d == 0 && threadIdx.x == 0) {
         st->next_index = 1ull;
         st->n_cur = nstart;
     }
-    if (ew32)  // (one block: the edges above are this block's own writes)
-        for (int d = 0; d < ndim; ++d) stage_axis(d, N, edges, ew32, map, tid, stride);
+    if (ew32) stage_axis(d, N, edges, ew32, map, threadIdx.x, blockDim.x);
 }
 
 __global__ void k_stage_grid(int ndim, int N, const double *edges, float2 *ew32, MapParams map)
@@ -557,10 +834,12 @@ __global__ void k_batch_reset(const BatchItem *items, const CombineArgs *cargs, 
     const int i = list ? list[blockIdx.x] : (int)blockIdx.x;
     const BatchItem &it = items[i];
     const int N = it.a.nbins, ndim = it.a.g.ndim;
-    for (int i = threadIdx.x; i < ndim * (N + 1); i += blockDim.x) {
-        const int k = i % (N + 1);
-        it.edges[i] = (double)k / (double)N;
-    }
+    // (each division once: FP64 divisions are slow here)
+    __shared__ double s_e[CV_MAX_BINS + 1];
+    for (int k = threadIdx.x; k <= N; k += blockDim.x) s_e[k] = (double)k / (double)N;
+    __syncthreads();
+    for (int d = 0; d < ndim; ++d)
+        for (int k = threadIdx.x; k <= N; k += blockDim.x) it.edges[(size_t)d * (N + 1) + k] = s_e[k];
     if (it.H)
         for (int i = threadIdx.x; i < ndim * N; i += blockDim.x) it.H[i] = 0.0;
     if (it.ew32) {
@@ -591,9 +870,9 @@ __global__ void __launch_bounds__(256) k_batch_refine(const BatchItem *items, co
         pa.part_nh = tp.stride;
         pa.part_f32 = 1;
         pa.part_slots = 1;
-        refine_axis(ax.y, it.a.nbins, it.H, it.edges, 0, it.ew32, &it.a.map, &pa);
+        refine_axis<kGroupBytesBatch>(ax.y, it.a.nbins, it.H, it.edges, 0, it.ew32, &it.a.map, &pa, nullptr);
     } else {
-        refine_axis(ax.y, it.a.nbins, it.H, it.edges, 1, it.ew32, &it.a.map);
+        refine_axis<kGroupBytesBatch>(ax.y, it.a.nbins, it.H, it.edges, 1, it.ew32, &it.a.map, nullptr, nullptr);
     }
 }
 
@@ -608,9 +887,9 @@ __global__ void k_batch_combine(const CombineArgs *cargs, const int *list, const
         CombineArgs B = A;
         B.part_S = part_S + (size_t)parts[i].row0 * (2 * CV_MAX_COMP);
         B.part_G = parts[i].count;
-        combine_iteration(B);
+        combine_iteration(B, nullptr);
     } else {
-        combine_iteration(A);
+        combine_iteration(A, nullptr);
     }
 }
 
@@ -658,7 +937,7 @@ cudaError_t launch_batch_combine(const CombineArgs *cargs, int count, cudaStream
 cudaError_t launch_reset(DevState *st, double *edges, double *H, int ndim, int nbins,
                          long long nstart, float2 *ew32, const MapParams &map, cudaStream_t s)
 {
-    k_reset<<<1, 256, 0, s>>>(st, edges, H, ndim, nbins, nstart, ew32, map);
+    k_reset<<<ndim, 256, 0, s>>>(st, edges, H, nbins, nstart, ew32, map);
     return cudaGetLastError();
 }
 
@@ -689,8 +968,8 @@ cudaError_t launch_refine_combine(int ndim, int nbins, double *H, double *edges,
                                   const CombineArgs &a, float2 *ew32, const MapParams &map,
                                   cudaStream_t s)
 {
-    // (with many block partials to add, a full CTA per axis: see
-    // sum_parts_axis; a few are summed by the threads of the bins)
+    // (with many block partials to add, a full CTA per axis: see sum_rows;
+    // a few are summed by the threads of the bins)
     const int threads = a.part_H && a.part_G >= 64 ? 1024 : refine_threads(nbins);
     k_refine_combine<<<ndim + 1, threads, 0, s>>>(ndim, nbins, H, edges, a, ew32, map);
     return cudaGetLastError();
