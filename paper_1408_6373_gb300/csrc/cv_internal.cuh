@@ -133,6 +133,20 @@ struct MapParams {
                                     // many steps (hist_phases); 0: shared-memory atomics
 };
 
+#if defined(__CUDACC__)
+// __double2float_rn from the bits for results that are normal (the
+// conversion instruction takes ~1000 cycles here); others go through it.
+__device__ __forceinline__ float round_f32(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)(b >> 52) & 2047;
+    if (e < 897 || e > 1150) return __double2float_rn(v);
+    const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);  // (to nearest, ties to even)
+    return __uint_as_float(((unsigned)(r >> 32) & 0x80000000u) |
+                           (((unsigned)(r >> 29) - 0xc0000000u) & 0x7fffffffu));  // (896 2^23, mod 2^32)
+}
+#endif
+
 // The FP32 sampling kernels' table entry of a bin with left edge e and
 // width w (both FP64), each half rounded once to binary32.  The kernels map
 // to the centred coordinate x - 1/2 (binary32 keeps absolute precision
@@ -140,13 +154,18 @@ struct MapParams {
 // [0, 1] values): x - 1/2 = fma(s w, f1, e - c w - 1/2), f1 the mantissa
 // construction of the fraction, c = 2^G and s = N for the power-of-two map,
 // c = s = 1 for the general one (where the kernel multiplies J by N).
+// (c w and s w are exact: powers of two.)
 __host__ __device__ __forceinline__ float2 grid_entry_f32(double e, double w, int N, const MapParams &m)
 {
+#if defined(__CUDA_ARCH__)
+    // the powers of two from their bits: an FP64 conversion or product is a
+    // long instruction here
+    const double c = __hiloint2double(m.pow2 ? (1023 + m.G) << 20 : 1023 << 20, 0);
+    const float s = m.pow2 ? (float)N : 1.0f;
+    return make_float2(round_f32(__fma_rn(-c, w, e) - 0.5), s * round_f32(w));
+#else
     const double c = m.pow2 ? (double)(1 << m.G) : 1.0;
     const double s = m.pow2 ? (double)N : 1.0;
-#if defined(__CUDA_ARCH__)
-    return make_float2(__double2float_rn(e - c * w - 0.5), __double2float_rn(s * w));
-#else
     return make_float2((float)(e - c * w - 0.5), (float)(s * w));
 #endif
 }

@@ -119,6 +119,18 @@ __device__ __forceinline__ unsigned long long shr64(unsigned long long v, int n)
     return n > 63 ? 0ull : v >> n;
 }
 
+// s + n for finite s >= 0 and its compensation |n| << s, from the bits (a
+// conversion to FP64 takes ~1000 cycles here).
+__device__ __forceinline__ Wide wide_of(float s, float n)
+{
+    const unsigned bs = (unsigned)max(__float_as_int(s), 0), bn = __float_as_uint(n);
+    const int es = (int)(bs >> 23), en = (int)(bn >> 23) & 255;
+    const unsigned long long ms = (unsigned long long)(es ? (bs & 0x7fffffu) | 0x800000u : bs) << 39;
+    const unsigned long long mn = (unsigned long long)(en ? (bn & 0x7fffffu) | 0x800000u : bn & 0x7fffffu) << 39;
+    const unsigned long long a = shr64(mn, max(es, 1) - max(en, 1));
+    return normalised(ms ? (bn >> 31 ? ms - a : ms + a) : 0ull, max(es, 1) - 189);
+}
+
 // 2^126 / m for a mantissa m (top bit set), to about 2^-60 of it: the
 // special-function unit's reciprocal y, then y (1 + e + e^2) with the exact
 // residual e = 1 - m y (Newton's iteration and its next term).
@@ -313,8 +325,6 @@ __device__ __forceinline__ float2 group_peer(const float2 &a, int o)
     return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
 }
 __device__ __forceinline__ double group_peer(const double &a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-__device__ __forceinline__ double group_value(const float2 &a) { return (double)a.x + (double)a.y; }
-__device__ __forceinline__ double group_value(const double &a) { return a; }
 
 template <int V>
 struct Sum64 {
@@ -331,9 +341,9 @@ struct Sum64 {
     }
 };
 
-// Space of the row groups' sums of a CTA of 1024 threads, and of one of 256
+// Space of the row groups' sums of a CTA of 512 threads, and of one of 256
 // (then the bins' prefix sums, weights and reciprocals).
-constexpr int kGroupBytes = 4352 * 8, kGroupBytesBatch = 1152 * 8;
+constexpr int kGroupBytes = 2304 * 8, kGroupBytesBatch = 1152 * 8;
 static_assert(kGroupBytesBatch >= (3 * CV_MAX_BINS + 1) * 8, "the bins' 64-bit values fit");
 
 // The sums over the G partial rows of one axis (first row P, row stride nh)
@@ -347,27 +357,28 @@ static_assert(kGroupBytesBatch >= (3 * CV_MAX_BINS + 1) * 8, "the bins' 64-bit v
 // FP32 (FP64 throughput is a small fraction of it here).  Called by every
 // thread of the CTA; synchronises before it returns.
 template <int GROUP, typename T, template <int> class S, typename E, int V>
-__device__ __forceinline__ void sum_rows(const CombineArgs *pa, int d, int N, unsigned char *raw, double *sH,
-                                         const MapParams *map)
+__device__ __forceinline__ void sum_rows(const CombineArgs *pa, int d, int N, unsigned c32, unsigned char *raw,
+                                         E *sums, const MapParams *map)
 {
-    // (the sums first, converted by the bins' warps alone: an FP64
-    // instruction of each of 32 warps takes 512 cycles)
-    E *sums = reinterpret_cast<E *>(sH);
     E *grp = reinterpret_cast<E *>(raw);
     const int G = pa->part_G;
     const size_t nh = (size_t)pa->part_nh;
-    // threads per bin, and a group stride that keeps their reads apart in
-    // the banks
-    const int lT = min(5, 31 - __clz((int)blockDim.x / N));
+    // Threads per bin (2^lT) and a group stride that keeps their reads apart
+    // in the banks.  FP64 additions cost 16 cycles of the SM per warp, so
+    // FP64 rows take at most eight groups.  (c32 = ceil(2^32 / N): quotients
+    // of values below 2^16 by N.)
+    const int lT = min(sizeof(T) == 8 ? 3 : 5, 31 - __clz((int)__umulhi(blockDim.x, c32)));
     const int T2 = 1 << lT;
     const int stride = ((N + 15) & ~15) + (lT >= 4 ? 1 : 16 >> lT);
     const int cols = N / V;
-    int R = min(min((int)blockDim.x / cols, GROUP / (int)(sizeof(E) * stride)), G);
-    const int t = threadIdx.x, r = t / cols, q = t - r * cols;
+    int R = min((int)__umulhi(blockDim.x * V, c32), G);
+    if (sizeof(T) == 8) R = min(R, 8);
+    if (N < 64) R = min(R, GROUP / (int)(sizeof(E) * stride));
+    const int t = threadIdx.x, r = (int)__umulhi((unsigned)t * V, c32), q = t - r * cols;
     if (r < R) {
         S<V> s;
         s.clear();
-        const T *p = static_cast<const T *>(pa->part_H) + (size_t)d * N + (size_t)q * V;
+        const T *p = static_cast<const T *>(pa->part_H) + (size_t)d * N + (size_t)(q * V);
         int b = r;
         for (; b + 7 * R < G; b += 8 * R) {
             T v[8][V];
@@ -422,11 +433,6 @@ __device__ __forceinline__ void sum_rows(const CombineArgs *pa, int d, int N, un
     // permuted store here costs nothing)
     if (k < N && j == 0) sums[sizeof(T) == 4 && pa->part_slots ? bin_of_slot(k, *map) : k] = s;
     __syncthreads();
-    if constexpr (sizeof(T) == 4) {
-        // (each thread its own slot)
-        if (t < N) sH[t] = group_value(sums[t]);
-        __syncthreads();
-    }
 }
 
 // Refine axis `d` of the grid in place, one CTA of at least N threads, all
@@ -440,7 +446,10 @@ __device__ void refine_axis(int d, int N, double *H, double *edges, int zero_his
     double *e = edges + (size_t)d * (N + 1);
     __shared__ __align__(16) unsigned char grp_raw[GROUP];
     __shared__ LogTable s_log;
-    __shared__ double sH[CV_MAX_BINS], se[CV_MAX_BINS + 1], sdw[CV_MAX_BINS];
+    __shared__ __align__(8) unsigned char sH_raw[CV_MAX_BINS * 8];  // the bins' sums: float2 or double
+    __shared__ double se[CV_MAX_BINS + 1], sdw[CV_MAX_BINS];
+    __shared__ unsigned long long hm[CV_MAX_BINS];                  // ... as Wide
+    __shared__ int he[CV_MAX_BINS];
     unsigned long long *sC = reinterpret_cast<unsigned long long *>(grp_raw);  // (after the row sums)
     unsigned long long *sR = sC + CV_MAX_BINS + 1, *sI = sR + CV_MAX_BINS;
     __shared__ unsigned long long wm[8], wt[8];
@@ -465,18 +474,19 @@ __device__ void refine_axis(int d, int N, double *H, double *edges, int zero_his
             lc[i] = g_log.c[at];
         }
     }
-    if (pa && pa->part_H) {
-        if (pa->part_f32) {
-            if (N % 4 == 0) sum_rows<GROUP, float, Sum32, float2, 4>(pa, d, N, grp_raw, sH, map);
-            else if (N % 2 == 0) sum_rows<GROUP, float, Sum32, float2, 2>(pa, d, N, grp_raw, sH, map);
-            else sum_rows<GROUP, float, Sum32, float2, 1>(pa, d, N, grp_raw, sH, map);
-        } else {
-            if (N % 2 == 0) sum_rows<GROUP, double, Sum64, double, 2>(pa, d, N, grp_raw, sH, map);
-            else sum_rows<GROUP, double, Sum64, double, 1>(pa, d, N, grp_raw, sH, map);
-        }
+    const unsigned q32 = 0xffffffffu / (unsigned)N, c32 = q32 + 1u;  // (c32 = ceil(2^32 / N))
+    const bool f32 = pa && pa->part_H && pa->part_f32;
+    if (f32) {
+        float2 *sums = reinterpret_cast<float2 *>(sH_raw);
+        if (N % 4 == 0) sum_rows<GROUP, float, Sum32, float2, 4>(pa, d, N, c32, grp_raw, sums, map);
+        else if (N % 2 == 0) sum_rows<GROUP, float, Sum32, float2, 2>(pa, d, N, c32, grp_raw, sums, map);
+        else sum_rows<GROUP, float, Sum32, float2, 1>(pa, d, N, c32, grp_raw, sums, map);
+    } else if (pa && pa->part_H) {
+        double *sums = reinterpret_cast<double *>(sH_raw);
+        if (N % 2 == 0) sum_rows<GROUP, double, Sum64, double, 2>(pa, d, N, c32, grp_raw, sums, map);
+        else sum_rows<GROUP, double, Sum64, double, 1>(pa, d, N, c32, grp_raw, sums, map);
     } else {
-        if (k < N) sH[k] = Hd[k];
-        __syncthreads();
+        if (k < N) reinterpret_cast<double *>(sH_raw)[k] = Hd[k];
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -488,28 +498,42 @@ __device__ void refine_axis(int d, int N, double *H, double *edges, int zero_his
     }
     // (whole warps leave: the barriers below count the others)
     if (!on || warp >= max(nw, 4)) return;
-    // 2^64 / N, at most N too small, from one 32-bit division
-    const unsigned q32 = 0xffffffffu / (unsigned)N;
+    // 2^64 / N, at most N too small
     const unsigned long long invN = ((unsigned long long)q32 << 32) + (unsigned long long)(0u - q32 * (unsigned)N) * q32;
     if (k < N) {
         se[k] = e0;
         sdw[k] = e1 - e0;
         if (k == N - 1) se[N] = e1;
     }
-    const double hk = k < N ? sH[k] : 0.0;
-    const int any_bad = __syncthreads_or(k < N && !isfinite(hk));
-    const int any_nz = __syncthreads_or(hk != 0.0);
+    // (each thread reads what it or, before a barrier, another thread wrote)
+    Wide hk{0, -100000};
+    bool finite = true;
+    if (k < N) {
+        if (f32) {
+            const float2 v = reinterpret_cast<const float2 *>(sH_raw)[k];
+            finite = isfinite(v.x + v.y);
+            hk = wide_of(v.x, v.y);
+        } else {
+            const double v = reinterpret_cast<const double *>(sH_raw)[k];
+            finite = isfinite(v);
+            hk = wide_of(v);
+        }
+        hm[k] = hk.m;
+        he[k] = hk.e;
+    }
+    const int any_bad = __syncthreads_or(!finite);
+    const int any_nz = __syncthreads_or(hk.m != 0ull);
     const bool act = warp < nw;  // (the other warps only meet the barriers)
     if (!any_bad && any_nz) {
         // smoothing over the neighbours, six times the mean: 2 (a + b + c)
         // inside, 3 (a + b) at the ends (an even histogram stays exactly even)
         Wide h{0, -100000};
         if (k < N) {
-            const Wide b = wide_of(hk);
-            const Wide a = k > 0 ? wide_of(sH[k - 1]) : Wide{0, -100000};
-            const Wide c = k < N - 1 ? wide_of(sH[k + 1]) : Wide{0, -100000};
-            const int E = max(b.e, max(a.e, c.e));
-            const unsigned long long v = shr64(a.m, 4 + E - a.e) + shr64(b.m, 4 + E - b.e) + shr64(c.m, 4 + E - c.e);
+            const Wide a = k > 0 ? Wide{hm[k - 1], he[k - 1]} : Wide{0, -100000};
+            const Wide c = k < N - 1 ? Wide{hm[k + 1], he[k + 1]} : Wide{0, -100000};
+            const int E = max(hk.e, max(a.e, c.e));
+            const unsigned long long v =
+                shr64(a.m, 4 + E - a.e) + shr64(hk.m, 4 + E - hk.e) + shr64(c.m, 4 + E - c.e);
             h = normalised((k > 0 && k < N - 1 ? 2ull : 3ull) * v, E);
         }
         // s = sum_k h_k: every warp at its own largest exponent, then the
@@ -578,10 +602,10 @@ __device__ void refine_axis(int d, int N, double *H, double *edges, int zero_his
             // product with ceil(2^32 / N))
             unsigned long long qn = __umul64hi(total, invN);
             unsigned rem = (unsigned)(total - qn * (unsigned)N);
-            const unsigned more = __umulhi(rem, q32 + 1u);
+            const unsigned more = __umulhi(rem, c32);
             qn += more;
             rem -= more * (unsigned)N;
-            const unsigned long long t = (unsigned long long)k * qn + __umulhi((unsigned)k * rem, q32 + 1u);
+            const unsigned long long t = (unsigned long long)k * qn + __umulhi((unsigned)k * rem, c32);
             // largest j in [0, N-1] with C_j <= t (then C_(j+1) > t, since t <
             // C_N), by quarters: the three probes of a step load together
             int lo = 0, len = N;  // the answer is in [lo, lo + len)
@@ -791,7 +815,7 @@ __device__ void combine_iteration(const CombineArgs &A, const int *active)
 // One Vegas iteration after its sampling pass: blocks 0..ndim-1 refine one
 // axis each from the histogram (and clear it), block ndim combines the
 // iteration.  Writes nothing unless the sampling launch before it ran.
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(512)
 k_refine_combine(int ndim, int N, double *H, double *edges, const CombineArgs A, float2 *ew32, MapParams map)
 {
     const int d = (int)blockIdx.x;
@@ -968,9 +992,11 @@ cudaError_t launch_refine_combine(int ndim, int nbins, double *H, double *edges,
                                   const CombineArgs &a, float2 *ew32, const MapParams &map,
                                   cudaStream_t s)
 {
-    // (with many block partials to add, a full CTA per axis: see sum_rows;
-    // a few are summed by the threads of the bins)
-    const int threads = a.part_H && a.part_G >= 64 ? 1024 : refine_threads(nbins);
+    // (with many block partials to add, a CTA of 512 threads per axis: see
+    // sum_rows -- 1024 hold no more rows in flight than L2 delivers, and add
+    // their groups' sums for longer, 10.3 against 8.3 us a launch for 64 bins;
+    // a few rows are summed by the threads of the bins)
+    const int threads = a.part_H && a.part_G >= 64 ? 512 : refine_threads(nbins);
     k_refine_combine<<<ndim + 1, threads, 0, s>>>(ndim, nbins, H, edges, a, ew32, map);
     return cudaGetLastError();
 }
