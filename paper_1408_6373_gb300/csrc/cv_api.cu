@@ -3123,6 +3123,7 @@ struct SuaveMem {
 __global__ void k_suave_prep(const SuaveEntry *E, const BatchItem *items, const double *dh_edges, int ndim,
                              int N, long long nnew, int *counter)
 {
+    wait_for_previous();
     const SuaveEntry e = E[blockIdx.x];
     const BatchItem &it = items[e.region];
     const int ge = ndim * (N + 1);
@@ -3147,6 +3148,7 @@ __global__ void k_suave_prep(const SuaveEntry *E, const BatchItem *items, const 
 __global__ void k_suave_gather(const SuaveEntry *E, const BatchItem *items, double *dh_S, double *dh_edges,
                                double *dh_fluct, int ndim, int N, int refined, double flatness)
 {
+    wait_for_previous();
     const int r = E[blockIdx.x].region;
     const BatchItem &it = items[r];
     const int ge = ndim * (N + 1);
@@ -3239,8 +3241,8 @@ int suave_pass_batched(cv_ctx *ctx, const cv_genz *g, int N, long long nnew, con
     const cudaStream_t s = ctx->stream;
     CV_CUDA(ctx, cudaMemcpyAsync(m.d_stage, m.h_stage, bytes, cudaMemcpyHostToDevice, s));
     const SuaveEntry *dE = reinterpret_cast<const SuaveEntry *>(m.d_stage);
-    k_suave_prep<<<(unsigned)nl, 256, 0, s>>>(dE, m.d_items, m.dh_edges, ndim, N, nnew, m.d_counter);
-    CV_CUDA(ctx, cudaGetLastError());
+    CV_CUDA(ctx, launch_kernel(k_suave_prep, (int)nl, 256, 0, s, dE, m.d_items, m.dh_edges, ndim, N, nnew,
+                               m.d_counter));
     BatchSampleArgs a;
     a.items = m.d_items;
     a.tiles = reinterpret_cast<const Tile *>(m.d_stage + off_t);
@@ -3252,9 +3254,8 @@ int suave_pass_batched(cv_ctx *ctx, const cv_genz *g, int N, long long nnew, con
     CV_CUDA(ctx, dispatch_batch_sample(ndim, m.pow2, a, m.grid < nt ? m.grid : nt, s));
     if (refine)
         CV_CUDA(ctx, launch_batch_refine(m.d_items, reinterpret_cast<const int2 *>(m.d_stage + off_a), naxes, s));
-    k_suave_gather<<<(unsigned)nl, 256, 0, s>>>(dE, m.d_items, m.dh_S, m.dh_edges, m.dh_fluct, ndim, N,
-                                                 refine ? 1 : 0, flatness);
-    CV_CUDA(ctx, cudaGetLastError());
+    CV_CUDA(ctx, launch_kernel(k_suave_gather, (int)nl, 256, 0, s, dE, m.d_items, m.dh_S, m.dh_edges, m.dh_fluct,
+                               ndim, N, refine ? 1 : 0, flatness));
     CV_CUDA(ctx, cudaStreamSynchronize(s));
     suave_read(g, N, nnew, list, refine, flatness, m, R);
     return CV_OK;

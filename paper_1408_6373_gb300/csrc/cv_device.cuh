@@ -1052,6 +1052,7 @@ template <int NDIM, typename Real, bool POW2, class I>
 __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
 {
     using W = typename Word<Real>::type;
+    wait_for_previous();
     unsigned long long start;
     long long n;
     if (A.st) {
@@ -1327,6 +1328,7 @@ template <int NDIM, bool POW2>
 __global__ void __launch_bounds__(kBlock, (kMinBlocks<NDIM, float>))
 k_batch_sample(const BatchSampleArgs B)
 {
+    wait_for_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int stride = B.stride;
     Smem<float> sm;
@@ -1598,6 +1600,7 @@ template <int NDIM, int L>
 __global__ void __launch_bounds__(kBlock, (kMinBlocks<NDIM, float>))
 k_mat_store(const __grid_constant__ SampleArgs<float> A)
 {
+    wait_for_previous();
     using P = Pow2Map<L>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned sx0[kWarpsPerBlock][NDIM][32];
@@ -1903,6 +1906,7 @@ template <int NDIM, int L>
 __global__ void __launch_bounds__(kBlock, kMatAccumBlocks)
 k_mat_accum(const __grid_constant__ SampleArgs<float> A)
 {
+    wait_for_previous();
     using P = Pow2Map<L>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int ncomp = A.g.ncomp;
@@ -2038,6 +2042,7 @@ template <int NDIM, typename Real, bool AOS>
 __global__ void __launch_bounds__(kBlock)
 k_genz_points(const __grid_constant__ GenzParams<Real> g, const Real *x, Real *f, long long n, long long ld)
 {
+    wait_for_previous();
     if constexpr (sizeof(Real) == 4 && !AOS) {
         genz_points_f32<NDIM, RuntimeIntegrand<float>>(g, x, f, n, ld);
         return;
@@ -2076,6 +2081,7 @@ __global__ void __launch_bounds__(kBlock)
 k_sobol(unsigned long long start, long long n, int shift, const __grid_constant__ PointArgs P,
         unsigned long long *Y)
 {
+    wait_for_previous();
     const int lane = threadIdx.x & 31;
     const unsigned long long qa = start >> 5;
     const unsigned long long end = start + (unsigned long long)n;
@@ -2126,14 +2132,13 @@ cudaError_t launch_sample(const SampleArgs<Real> &a, int grid, cudaStream_t s)
     // (sample_occupancy, always called first, sets the shared-memory limit)
     const size_t smem = sample_smem_bytes(NDIM, a.nbins, sizeof(Real) == 8, a.map.priv != 0);
     if (a.gen == kGenPseudo) {
-        k_sample_pseudo<NDIM, Real><<<grid, kBlock, smem, s>>>(a);
+        return launch_kernel(k_sample_pseudo<NDIM, Real>, grid, kBlock, smem, s, a);
     } else if constexpr (sizeof(Real) == 4) {
-        if (a.map.pow2) k_sample<NDIM, float, true><<<grid, kBlock, smem, s>>>(a);
-        else k_sample<NDIM, float, false><<<grid, kBlock, smem, s>>>(a);
+        return launch_kernel(a.map.pow2 ? k_sample<NDIM, float, true> : k_sample<NDIM, float, false>, grid, kBlock,
+                             smem, s, a);
     } else {
-        k_sample<NDIM, double, false><<<grid, kBlock, smem, s>>>(a);
+        return launch_kernel(k_sample<NDIM, double, false>, grid, kBlock, smem, s, a);
     }
-    return cudaGetLastError();
 }
 
 template <int NDIM, typename Real>
@@ -2169,8 +2174,7 @@ template <int NDIM, bool POW2>
 cudaError_t launch_batch_sample(const BatchSampleArgs &b, int grid, cudaStream_t s)
 {
     // (batch_occupancy, always called first, sets the shared-memory limit)
-    k_batch_sample<NDIM, POW2><<<grid, kBlock, batch_smem_bytes(NDIM, b.stride), s>>>(b);
-    return cudaGetLastError();
+    return launch_kernel(k_batch_sample<NDIM, POW2>, grid, kBlock, batch_smem_bytes(NDIM, b.stride), s, b);
 }
 
 template <int NDIM>
@@ -2203,8 +2207,7 @@ static cudaError_t launch_mat_lean(const SampleArgs<float> &a, int grid, cudaStr
         cudaError_t e = cudaFuncSetAttribute(k_mat_store<NDIM, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         *grid_used = grid;
-        k_mat_store<NDIM, L><<<grid, kBlock, smem, s>>>(a);
-        return cudaGetLastError();
+        return launch_kernel(k_mat_store<NDIM, L>, grid, kBlock, smem, s, a);
     }
     // (the width table, the warps' histogram copies, 8N bytes to align the
     // table, the warps' value rings)
@@ -2226,8 +2229,7 @@ static cudaError_t launch_mat_lean(const SampleArgs<float> &a, int grid, cudaStr
     if (grid > sms * occ) grid = sms * occ;
     if (a.part_S && grid > a.part_G) return cudaErrorInvalidValue;  // (partial rows for every block)
     *grid_used = grid;
-    k_mat_accum<NDIM, L><<<grid, kBlock, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_kernel(k_mat_accum<NDIM, L>, grid, kBlock, smem, s, a);
 }
 
 template <int NDIM, typename Real, bool POW2, int MODE>
@@ -2252,8 +2254,7 @@ static cudaError_t launch_matpass_v(const SampleArgs<Real> &a, int grid, cudaStr
     if (e != cudaSuccess) return e;
     if (a.part_S && grid > a.part_G) return cudaErrorInvalidValue;
     *grid_used = grid;
-    k_matpass<NDIM, Real, POW2, MODE><<<grid, kBlock, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_kernel(k_matpass<NDIM, Real, POW2, MODE>, grid, kBlock, smem, s, a);
 }
 
 template <int NDIM, typename Real, int MODE>
@@ -2269,8 +2270,7 @@ template <int NDIM, typename Real, bool AOS>
 cudaError_t launch_genz_points(const GenzParams<Real> &g, const Real *x, Real *f, long long n,
                                long long ld, int grid, cudaStream_t s)
 {
-    k_genz_points<NDIM, Real, AOS><<<grid, kBlock, 0, s>>>(g, x, f, n, ld);
-    return cudaGetLastError();
+    return launch_kernel(k_genz_points<NDIM, Real, AOS>, grid, kBlock, 0, s, g, x, f, n, ld);
 }
 
 template <int NDIM, typename W>
@@ -2278,8 +2278,7 @@ cudaError_t launch_sobol(unsigned long long start, long long n, int bits, const 
                          unsigned long long *Y, int grid, cudaStream_t s)
 {
     const int shift = (int)(8 * sizeof(W)) - bits;
-    k_sobol<NDIM, W><<<grid, kBlock, 0, s>>>(start, n, shift, pa, Y);
-    return cudaGetLastError();
+    return launch_kernel(k_sobol<NDIM, W>, grid, kBlock, 0, s, start, n, shift, pa, Y);
 }
 
 #endif  // !__CUDACC_RTC__

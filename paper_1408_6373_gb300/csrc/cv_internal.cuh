@@ -13,6 +13,55 @@
 
 namespace cv {
 
+// ---- launches that follow one another in a stream
+// A kernel launched after another in a stream costs 2 to 4 us besides its
+// work on this system, and ends on a multiple of 2.05 us; with programmatic
+// stream serialization (the launch is set up while the kernel before it still
+// runs) 0.6 us, as between the nodes of a graph.  (100 kernels of 2.6 us on
+// 152 CTAs: 5.1 us each plain, 3.1 us so.)  Every kernel of the library is
+// launched that way and first waits for the work before it, before any
+// access to memory; none signals early, so the next kernel's CTAs take no
+// place until the last CTA leaves.
+#if defined(__CUDACC__)
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
+#if !defined(__CUDACC_RTC__)
+// (a launch that is being captured stays plain: a graph's nodes gain nothing)
+inline bool chains_launches(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st == cudaStreamCaptureStatusNone;
+}
+inline cudaError_t launch_raw(const void *kernel, int grid, int block, size_t smem, cudaStream_t s, void **args)
+{
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = chains_launches(s) ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, args);
+    if (e != cudaSuccess) cudaGetLastError();  // (returned, not left for a later call)
+    return e;
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args)
+{
+    return [&](P... p) {
+        void *ptr[] = {(void *)&p...};
+        return launch_raw((const void *)kernel, grid, block, smem, s, ptr);
+    }(args...);
+}
+#endif
+
 constexpr int kWarp = 32;
 constexpr int kBlock = 256;                 // threads per sampling block
 constexpr int kWarpsPerBlock = kBlock / kWarp;

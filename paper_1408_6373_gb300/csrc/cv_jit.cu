@@ -157,6 +157,7 @@ std::string points_source(const GenzParams<float> &g, int ndim)
     s += "extern \"C\" __global__ void __launch_bounds__(" + std::to_string(kBlock) +
          ") cv_jit_points(const __grid_constant__ cv::GenzParams<float> g, const float *x, float *f, "
          "long long n, long long ld)\n{\n";
+    s += "    cv::wait_for_previous();\n";
     s += "    cv::genz_points_f32<" + std::to_string(ndim) + ", cv::JitIntegrand>(g, x, f, n, ld);\n}\n";
     return s;
 }
@@ -310,13 +311,13 @@ cudaError_t launch_jit_points(const JitKernel &k, const GenzParams<float> &g, co
                               long long ld, int grid, cudaStream_t s)
 {
     void *args[5] = {const_cast<GenzParams<float> *>(&g), &x, &f, &n, &ld};
-    return cudaLaunchKernel((const void *)k.kernel, dim3(grid), dim3(kBlock), args, 0, s);
+    return launch_raw((const void *)k.kernel, grid, kBlock, 0, s, args);
 }
 
 cudaError_t launch_jit_sample(const JitKernel &k, const SampleArgs<float> &a, int grid, cudaStream_t s)
 {
     void *args[1] = {const_cast<SampleArgs<float> *>(&a)};
-    return cudaLaunchKernel((const void *)k.kernel, dim3(grid), dim3(kBlock), args, k.smem, s);
+    return launch_raw((const void *)k.kernel, grid, kBlock, k.smem, s, args);
 }
 
 }  // namespace cv

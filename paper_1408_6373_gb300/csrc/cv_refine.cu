@@ -640,6 +640,7 @@ __device__ void refine_axis(int d, int N, double *H, double *edges, int zero_his
 // the 8 results are added in j order -- a fixed order, so deterministic.
 __global__ void __launch_bounds__(256) k_add_parts(const void *part_H, int G, int f32, int nh, double *H)
 {
+    wait_for_previous();
     __shared__ double part[8][32];
     const int bin = threadIdx.x & 31, j = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + bin;
@@ -671,6 +672,7 @@ __global__ void __launch_bounds__(256) k_add_parts(const void *part_H, int G, in
 
 __global__ void __launch_bounds__(256) k_refine(int N, double *H, double *edges)
 {
+    wait_for_previous();
     refine_axis<kGroupBytesBatch>(blockIdx.x, N, H, edges, 0, nullptr, nullptr, nullptr, nullptr);
 }
 
@@ -818,6 +820,7 @@ __device__ void combine_iteration(const CombineArgs &A, const int *active)
 __global__ void __launch_bounds__(512)
 k_refine_combine(int ndim, int N, double *H, double *edges, const CombineArgs A, float2 *ew32, MapParams map)
 {
+    wait_for_previous();
     const int d = (int)blockIdx.x;
     if (d < ndim) refine_axis<kGroupBytes>(d, N, H, edges, 1, ew32, &map, &A, &A.st->pass_active);
     else combine_iteration(A, &A.st->pass_active);
@@ -829,6 +832,7 @@ k_refine_combine(int ndim, int N, double *H, double *edges, const CombineArgs A,
 // for 30 axes of 256 bins in one CTA, 4 us so).
 __global__ void k_reset(DevState *st, double *edges, double *H, int N, long long nstart, float2 *ew32, MapParams map)
 {
+    wait_for_previous();
     const int d = blockIdx.x;
     double *e = edges + (size_t)d * (N + 1);
     for (int k = threadIdx.x; k <= N; k += blockDim.x) e[k] = (double)k / (double)N;
@@ -847,6 +851,7 @@ __global__ void k_reset(DevState *st, double *edges, double *H, int N, long long
 
 __global__ void k_stage_grid(int ndim, int N, const double *edges, float2 *ew32, MapParams map)
 {
+    wait_for_previous();
     stage_axis(blockIdx.x, N, edges, ew32, map, threadIdx.x, blockDim.x);
 }
 
@@ -855,6 +860,7 @@ __global__ void k_stage_grid(int ndim, int N, const double *edges, float2 *ew32,
 // its stop flag is only ever set by a later combine launch.
 __global__ void k_batch_reset(const BatchItem *items, const CombineArgs *cargs, const int *list)
 {
+    wait_for_previous();
     const int i = list ? list[blockIdx.x] : (int)blockIdx.x;
     const BatchItem &it = items[i];
     const int N = it.a.nbins, ndim = it.a.g.ndim;
@@ -882,6 +888,7 @@ __global__ void k_batch_reset(const BatchItem *items, const CombineArgs *cargs, 
 __global__ void __launch_bounds__(256) k_batch_refine(const BatchItem *items, const int2 *axes,
                                                       const TileParts *parts, const float *part_H)
 {
+    wait_for_previous();
     const int2 ax = axes[blockIdx.x];
     const BatchItem &it = items[ax.x];
     if (*(volatile const int *)&it.st->stopped) return;
@@ -903,6 +910,7 @@ __global__ void __launch_bounds__(256) k_batch_refine(const BatchItem *items, co
 __global__ void k_batch_combine(const CombineArgs *cargs, const int *list, const TileParts *parts,
                                 const double *part_S)
 {
+    wait_for_previous();
     const int i = list ? list[blockIdx.x] : (int)blockIdx.x;
     const CombineArgs &A = cargs[i];
     if (*(volatile const int *)&A.st->stopped) return;
@@ -921,14 +929,14 @@ cudaError_t launch_batch_reset(const BatchItem *items, const CombineArgs *cargs,
                                cudaStream_t s, const int *list)
 {
     if (count <= 0) return cudaSuccess;
-    k_batch_reset<<<count, 256, 0, s>>>(items, cargs, list);
-    return cudaGetLastError();
+    return launch_kernel(k_batch_reset, count, 256, 0, s, items, cargs, list);
 }
 
 // Copy the states of the listed integrals (null list: of all of them, in
 // order) into one contiguous array.
 __global__ void k_gather_states(const BatchItem *items, const int *list, DevState *out)
 {
+    wait_for_previous();
     const int *src = reinterpret_cast<const int *>(items[list ? list[blockIdx.x] : (int)blockIdx.x].st);
     int *dst = reinterpret_cast<int *>(out + blockIdx.x);
     for (int i = threadIdx.x; i < (int)(sizeof(DevState) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
@@ -938,38 +946,33 @@ cudaError_t launch_gather_states(const BatchItem *items, const int *list, int co
                                  cudaStream_t s)
 {
     if (count <= 0) return cudaSuccess;
-    k_gather_states<<<count, 32, 0, s>>>(items, list, out);
-    return cudaGetLastError();
+    return launch_kernel(k_gather_states, count, 32, 0, s, items, list, out);
 }
 
 cudaError_t launch_batch_refine(const BatchItem *items, const int2 *axes, int naxes, cudaStream_t s,
                                 const TileParts *parts, const float *part_H)
 {
     if (naxes <= 0) return cudaSuccess;
-    k_batch_refine<<<naxes, 256, 0, s>>>(items, axes, parts, part_H);
-    return cudaGetLastError();
+    return launch_kernel(k_batch_refine, naxes, 256, 0, s, items, axes, parts, part_H);
 }
 
 cudaError_t launch_batch_combine(const CombineArgs *cargs, int count, cudaStream_t s, const int *list,
                                  const TileParts *parts, const double *part_S)
 {
     if (count <= 0) return cudaSuccess;
-    k_batch_combine<<<count, 32, 0, s>>>(cargs, list, parts, part_S);
-    return cudaGetLastError();
+    return launch_kernel(k_batch_combine, count, 32, 0, s, cargs, list, parts, part_S);
 }
 
 cudaError_t launch_reset(DevState *st, double *edges, double *H, int ndim, int nbins,
                          long long nstart, float2 *ew32, const MapParams &map, cudaStream_t s)
 {
-    k_reset<<<ndim, 256, 0, s>>>(st, edges, H, nbins, nstart, ew32, map);
-    return cudaGetLastError();
+    return launch_kernel(k_reset, ndim, 256, 0, s, st, edges, H, nbins, nstart, ew32, map);
 }
 
 cudaError_t launch_stage_grid(int ndim, int nbins, const double *edges, float2 *ew32,
                               const MapParams &map, cudaStream_t s)
 {
-    k_stage_grid<<<ndim, 256, 0, s>>>(ndim, nbins, edges, ew32, map);
-    return cudaGetLastError();
+    return launch_kernel(k_stage_grid, ndim, 256, 0, s, ndim, nbins, edges, ew32, map);
 }
 
 // Threads of a refinement CTA: the bins rounded up to whole warps, at least
@@ -978,14 +981,12 @@ static int refine_threads(int nbins) { return nbins <= 64 ? 64 : (nbins + 31) / 
 
 cudaError_t launch_add_parts(const void *part_H, int G, int f32, int nh, double *H, cudaStream_t s)
 {
-    k_add_parts<<<(nh + 31) / 32, 256, 0, s>>>(part_H, G, f32, nh, H);
-    return cudaGetLastError();
+    return launch_kernel(k_add_parts, (nh + 31) / 32, 256, 0, s, part_H, G, f32, nh, H);
 }
 
 cudaError_t launch_refine(int ndim, int nbins, double *H, double *edges, cudaStream_t s)
 {
-    k_refine<<<ndim, refine_threads(nbins), 0, s>>>(nbins, H, edges);
-    return cudaGetLastError();
+    return launch_kernel(k_refine, ndim, refine_threads(nbins), 0, s, nbins, H, edges);
 }
 
 cudaError_t launch_refine_combine(int ndim, int nbins, double *H, double *edges,
@@ -997,8 +998,7 @@ cudaError_t launch_refine_combine(int ndim, int nbins, double *H, double *edges,
     // their groups' sums for longer, 10.3 against 8.3 us a launch for 64 bins;
     // a few rows are summed by the threads of the bins)
     const int threads = a.part_H && a.part_G >= 64 ? 512 : refine_threads(nbins);
-    k_refine_combine<<<ndim + 1, threads, 0, s>>>(ndim, nbins, H, edges, a, ew32, map);
-    return cudaGetLastError();
+    return launch_kernel(k_refine_combine, ndim + 1, threads, 0, s, ndim, nbins, H, edges, a, ew32, map);
 }
 
 }  // namespace cv
