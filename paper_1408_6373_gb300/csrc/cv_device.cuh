@@ -245,6 +245,15 @@ struct RuntimeIntegrand {
     __device__ __forceinline__ static int nbins(int n) { return n; }
 };
 
+// N = 2^L bins at compile time: the strides of the grid table and of the
+// histogram copies are then offsets in the instructions (the map's masks
+// stay launch constants: as immediates they cost more).
+template <int L>
+struct FixedBins : RuntimeIntegrand<float> {
+    __device__ __forceinline__ static int table(const MapParams &) { return L - 4; }
+    __device__ __forceinline__ static int nbins(int) { return 1 << L; }
+};
+
 // Pseudo-random points (Philox words per point instead of the Sobol
 // recurrence) with the integrand evaluated in the pass.
 template <typename Real>
@@ -1047,6 +1056,53 @@ __device__ __forceinline__ void last_block_sums(const double *part_S, unsigned *
     if (threadIdx.x == 0) *ticket = 0u;
 }
 
+// The block's sums (warp, then across the warps in FP64): its partial row,
+// or FP64 atomics.
+template <typename Real>
+__device__ __forceinline__ void block_sums(const SampleArgs<Real> &A, int ncomp, const Acc<Real> (&s1)[CV_MAX_COMP],
+                                           const Acc<Real> (&s2)[CV_MAX_COMP])
+{
+    __shared__ double red[kWarpsPerBlock][2 * CV_MAX_COMP];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int c = 0; c < CV_MAX_COMP; ++c) {
+        if (c < ncomp) {
+            const double a = warp_total(s1[c]);
+            const double b = warp_total(s2[c]);
+            if (lane == 0) {
+                red[warp][2 * c] = a;
+                red[warp][2 * c + 1] = b;
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * ncomp) {
+        double t = 0.0;
+        for (int w = 0; w < kWarpsPerBlock; ++w) t += red[w][threadIdx.x];
+        const int c = threadIdx.x >> 1;
+        if (A.part_S) A.part_S[blockIdx.x * (2 * CV_MAX_COMP) + threadIdx.x] = t;
+        else atomicAdd((threadIdx.x & 1) ? &A.S2[c] : &A.S1[c], t);
+    }
+}
+
+// The index range of a pass: the launch's, or the one the device state
+// decided on (then false once the run has stopped).
+template <typename Real>
+__device__ __forceinline__ bool pass_range(const SampleArgs<Real> &A, unsigned long long &start, long long &n)
+{
+    if (A.st) {
+        const int stopped = *(volatile const int *)&A.st->stopped;
+        if (blockIdx.x == 0 && threadIdx.x == 0) A.st->pass_active = stopped ? 0 : 1;
+        if (stopped) return false;
+        start = A.st->next_index;
+        n = A.st->n_cur;
+    } else {
+        start = A.start;
+        n = A.n;
+    }
+    return true;
+}
+
 // One fused sampling pass (the kernel body, shared by every specialisation).
 template <int NDIM, typename Real, bool POW2, class I>
 __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
@@ -1055,20 +1111,12 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
     wait_for_previous();
     unsigned long long start;
     long long n;
-    if (A.st) {
-        const int stopped = *(volatile const int *)&A.st->stopped;
-        if (blockIdx.x == 0 && threadIdx.x == 0) A.st->pass_active = stopped ? 0 : 1;
-        if (stopped) return;
-        start = A.st->next_index;
-        n = A.st->n_cur;
-    } else {
-        start = A.start;
-        n = A.n;
-    }
+    if (!pass_range(A, start, n)) return;
     const int N = I::nbins(A.nbins);
     const int ncomp = A.g.ncomp;
     // warp copies of the histogram for Sobol points when they fit
-    const bool priv = I::kGen != 2 && (sizeof(Real) == 4 ? I::priv(A.map) : A.map.priv != 0);
+    // (FP32 power-of-two passes whose copies do not fit: sample_pass_owner)
+    const bool priv = I::kGen != 2 && (sizeof(Real) == 4 ? (POW2 && I::kMode == 0) || I::priv(A.map) : A.map.priv != 0);
     const int hmode = !priv ? kHistBlock : (sizeof(Real) == 4 && POW2 ? kHistWarpPlain : kHistWarpPhased);
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1155,29 +1203,8 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
 
     if constexpr (I::kMode == 1) return;  // points stored: nothing to reduce
 
-    // Reduction: warp, then across the block's warps in FP64.
-    __shared__ double red[kWarpsPerBlock][2 * CV_MAX_COMP];
-    const int warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < CV_MAX_COMP; ++c) {
-        if (c < ncomp) {
-            const double a = warp_total(s1[c]);
-            const double b = warp_total(s2[c]);
-            if (lane == 0) {
-                red[warp][2 * c] = a;
-                red[warp][2 * c + 1] = b;
-            }
-        }
-    }
-    __syncthreads();
+    block_sums(A, ncomp, s1, s2);
     const bool parts = A.part_S != nullptr;
-    if (threadIdx.x < 2 * ncomp) {
-        double t = 0.0;
-        for (int w = 0; w < kWarpsPerBlock; ++w) t += red[w][threadIdx.x];
-        const int c = threadIdx.x >> 1;
-        if (parts) A.part_S[blockIdx.x * (2 * CV_MAX_COMP) + threadIdx.x] = t;
-        else atomicAdd((threadIdx.x & 1) ? &A.S2[c] : &A.S1[c], t);
-    }
     // (by bin: the FP64 atomics of a warp go to consecutive addresses,
     // which the L2 merges; every block flushes at about the same time)
     Real *ph = parts ? reinterpret_cast<Real *>(A.part_H) + (size_t)blockIdx.x * NDIM * N : nullptr;
@@ -1211,11 +1238,189 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
     if (parts && A.part_ticket) last_block_sums(A.part_S, A.part_ticket, A.S1, A.S2, ncomp);
 }
 
-template <int NDIM, typename Real, bool POW2>
+// The FP32 pass for N = 2^L >= 32 when the warps' histogram copies do not fit
+// (256 bins from 7 dimensions on, 128 from 22): one copy per block, and
+// every axis's row belongs to one warp, which alone updates it, without
+// atomics (a compare-and-swap loop on this GPU) and without conflicts.  The
+// block's eight warps evaluate eight consecutive 32-point blocks a round
+// (an aligned group), leave (J f_0)^2 of their points in shared memory, meet
+// at a barrier, and each warp then adds the 256 values to its axes' bins:
+// it walks those axes' words through the group by the Gray-code recurrence
+// itself, one XOR per block, so no word goes through shared memory.  Two
+// buffers of values, so one barrier a round.
+// 30 dimensions, 256 bins, 5e7 points: 1269 us (block atomics: 1740 us),
+// bound by instruction issue (668 instructions a block, 66% of the slots).
+template <int NDIM, class I>
+__device__ __forceinline__ void sample_pass_owner(const SampleArgs<float> &A)
+{
+    wait_for_previous();
+    unsigned long long start;
+    long long n;
+    if (!pass_range(A, start, n)) return;
+    const int N = I::nbins(A.nbins), ncomp = I::ncomp(A.g), li = I::table(A.map);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Smem<float> sm;
+    sm.stride = N;
+    sm.ew = align_table(smem_raw, N);
+    float *hist = reinterpret_cast<float *>(sm.ew + NDIM * N);
+    sm.h = hist;
+    float *sq = hist + NDIM * N;  // [2][kWarpsPerBlock][32]
+    for (int i = threadIdx.x; i < NDIM * N; i += blockDim.x) hist[i] = 0.0f;
+    if (A.ew32) {
+        for (int idx = threadIdx.x; idx < NDIM * N; idx += blockDim.x) sm.ew[idx] = A.ew32[idx];
+    } else {
+        stage_grid_f32(sm.ew, NDIM, N, N, A.edges, A.map);
+    }
+    set_addresses(sm, A.map.L);
+
+    // groups of eight blocks [ga, gb) cover the pass; a run of them per block
+    const unsigned long long end = start + (unsigned long long)n;
+    const unsigned long long ga = start >> 8, gb = n > 0 ? (end + 255ull) >> 8 : ga;
+    const unsigned long long per = (gb - ga + gridDim.x - 1) / gridDim.x;
+    const unsigned long long g0 = min(ga + blockIdx.x * per, gb);
+    const int rounds = (int)(min(g0 + per, gb) - g0);
+    Acc<float> s1[CV_MAX_COMP], s2[CV_MAX_COMP];
+    constexpr int kOwn = (NDIM + kWarpsPerBlock - 1) / kWarpsPerBlock;  // axes of a warp: warp, warp + 8, ...
+    unsigned X[NDIM];
+    sobol_skip<NDIM, unsigned>(X, g0 * 8ull + (unsigned)warp, lane, li);
+    if (A.gen == kGenScrambled) {
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d) X[d] ^= (unsigned)A.shift[d];
+    }
+    // this warp's axes' words at the group's first block, handed over through
+    // the buffer of squares (warp 0 holds block 0's)
+    unsigned O[kOwn];
+#pragma unroll
+    for (int j = 0; j < kOwn; ++j) {
+        __syncthreads();
+        if (warp == 0) {
+#pragma unroll
+            for (int w = 0; w < kWarpsPerBlock; ++w)
+                if (8 * j + w < NDIM) reinterpret_cast<unsigned *>(sq)[w * 32 + lane] = X[8 * j + w < NDIM ? 8 * j + w : 0];
+        }
+        __syncthreads();
+        O[j] = reinterpret_cast<unsigned *>(sq)[warp * 32 + lane];
+    }
+    __syncthreads();
+    // ... and the steps between a group's blocks as differences of a slot's
+    // byte offset in its row
+    auto own = [&](int j) { return min(warp + 8 * j, NDIM - 1); };
+    unsigned step[kOwn][3];
+#pragma unroll
+    for (int j = 0; j < kOwn; ++j) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) step[j][k] = (Dir<unsigned>::w(li, own(j), 5 + k) >> (32 - A.map.L)) << 2;
+    }
+
+    const int delay = I::delay(A.g);
+    Partial<float> P;
+    P.zero();
+    for (int r = 0; r < rounds; ++r) {
+        const unsigned long long group = g0 + (unsigned long long)r;
+        const unsigned long long i = group * 256ull + threadIdx.x;
+        const bool valid = i >= start && i < end;
+        float z[NDIM];
+        float J = 1.0f;
+        unsigned slot;
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d) z[d] = map_f32<true>(X[d], d, N, A.map, sm, J, slot);
+        if (delay) J += 0.0f * delay_chain<NDIM>(z, delay * ncomp);
+        if (!valid) J = 0.0f;  // (f is finite at every point of the block)
+        const float v0 = J * genz_f32<NDIM, 0, I>(A.g, z);
+        float *buf = sq + (r & 1) * kBlock;
+        buf[threadIdx.x] = v0 * v0;
+        const float f1 = ncomp > 1 ? genz_f32<NDIM, 1, I>(A.g, z) : 0.0f;
+        const float2 v01 = make_float2(v0, J * f1);
+        P.s1[0] = add2(P.s1[0], v01);
+        P.s2[0] = fma2(v01, v01, P.s2[0]);
+        if (ncomp > 2) {
+            const float f2 = genz_f32<NDIM, 2, I>(A.g, z);
+            const float f3 = ncomp > 3 ? genz_f32<NDIM, 3, I>(A.g, z) : 0.0f;
+            const float2 v23 = make_float2(J * f2, J * f3);
+            P.s1[1] = add2(P.s1[1], v23);
+            P.s2[1] = fma2(v23, v23, P.s2[1]);
+        }
+        if ((r + 1) % (int)kRun == 0 || r + 1 == rounds) {
+#pragma unroll
+            for (int c = 0; c < CV_MAX_COMP; ++c) {
+                if (c < ncomp) {
+                    s1[c].add(P.v1(c));
+                    s2[c].add(P.v2(c));
+                }
+            }
+            P.zero();
+        }
+        // the step from this group's blocks to the next group's (i + 256):
+        // Gray-code bits 7 and 8 + ctz(group + 1) flip
+        const int k = 8 + min(__ffsll((long long)(group + 1ull)) - 1, CV_SOBOL_BITS - 9);
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d) X[d] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
+        __syncthreads();
+        // the group's 256 values into this warp's axes: a row starts on a
+        // multiple of its size, so the step to the next block's slot is an
+        // XOR of the address itself
+        float h[kWarpsPerBlock];
+#pragma unroll
+        for (int w = 0; w < kWarpsPerBlock; ++w) h[w] = buf[w * 32 + lane];
+        unsigned at[kOwn];
+#pragma unroll
+        for (int j = 0; j < kOwn; ++j) {
+            const int d = own(j);
+            at[j] = __funnelshift_r(O[j], sm.h_hi + (unsigned)d, A.map.sA + 1u);
+            O[j] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
+        }
+#pragma unroll
+        for (int w = 0; w < kWarpsPerBlock; ++w) {
+            float v[kOwn];
+#pragma unroll
+            for (int j = 0; j < kOwn; ++j)
+                if (warp + 8 * j < NDIM) v[j] = lds_f(at[j]);
+#pragma unroll
+            for (int j = 0; j < kOwn; ++j) {
+                if (warp + 8 * j < NDIM) sts_f(at[j], v[j] + h[w]);
+                // (out of block w of the group: bits 4 and 5 + ctz(w + 1) flip)
+                if (w < 7) at[j] ^= step[j][w & 1 ? (w == 3 ? 2 : 1) : 0];
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    block_sums(A, ncomp, s1, s2);
+    const bool parts = A.part_S != nullptr;
+    float *ph = parts ? reinterpret_cast<float *>(A.part_H) + (size_t)blockIdx.x * NDIM * N : nullptr;
+    for (int idx = threadIdx.x; idx < NDIM * N; idx += blockDim.x) {
+        const int d = idx / N, b = idx - d * N;
+        const float v = hist[d * N + slot_of_bin(b, A.map)];
+        if (parts) ph[idx] = v;
+        else if (v != 0.0f) atomicAdd(&A.H[idx], (double)v);
+    }
+    if (parts && A.part_ticket) last_block_sums(A.part_S, A.part_ticket, A.S1, A.S2, ncomp);
+}
+
+template <int NDIM, int L>
+__global__ void __launch_bounds__(kBlock, (kMinBlocks<NDIM, float>))
+k_sample_owner(const __grid_constant__ SampleArgs<float> A)
+{
+    sample_pass_owner<NDIM, FixedBins<L>>(A);
+}
+
+// The fused pass on the general map (FP64, and FP32 for other bin counts) ...
+template <int NDIM, typename Real>
 __global__ void __launch_bounds__(kBlock, (kMinBlocks<NDIM, Real>))
 k_sample(const __grid_constant__ SampleArgs<Real> A)
 {
-    sample_pass<NDIM, Real, POW2, RuntimeIntegrand<Real>>(A);
+    sample_pass<NDIM, Real, false, RuntimeIntegrand<Real>>(A);
+}
+
+// ... and for N = 2^L, L = 5..8: bound by instruction issue (8 dimensions, 4
+// components, 1e7 points: 331 instructions a block, 70% of the slots, 126 us;
+// 347 and 134 us with the bin count a launch argument).
+template <int NDIM, int L>
+__global__ void __launch_bounds__(kBlock, (kMinBlocks<NDIM, float>))
+k_sample_pow2(const __grid_constant__ SampleArgs<float> A)
+{
+    sample_pass<NDIM, float, true, FixedBins<L>>(A);
 }
 
 // The pass with pseudo-random points (CV_PSEUDO), on the generic map.
@@ -2117,13 +2322,34 @@ k_sobol(unsigned long long start, long long n, int shift, const __grid_constant_
 
 // ------------------------------------------------------------ launchers
 #if !defined(__CUDACC_RTC__)
+using SampleFn32 = void (*)(SampleArgs<float>);
+
+// The FP32 kernel for N = 2^L bins (null: the map's choice of histogram is
+// not the one this dimension count is compiled for).
+template <int NDIM, int L>
+static SampleFn32 sample_fn_bins(bool priv)
+{
+    if constexpr (copies_fit(NDIM, 1 << L, false)) return priv ? k_sample_pow2<NDIM, L> : nullptr;
+    else return priv ? nullptr : k_sample_owner<NDIM, L>;
+}
+template <int NDIM>
+static SampleFn32 sample_fn_pow2(int L, bool priv)
+{
+    switch (L) {
+    case 5: return sample_fn_bins<NDIM, 5>(priv);
+    case 6: return sample_fn_bins<NDIM, 6>(priv);
+    case 7: return sample_fn_bins<NDIM, 7>(priv);
+    case 8: return sample_fn_bins<NDIM, 8>(priv);
+    default: return nullptr;
+    }
+}
+
 template <int NDIM, typename Real>
-static void *sample_fn(bool pow2)
+static const void *sample_fn(const MapParams &m)
 {
     if constexpr (sizeof(Real) == 4)
-        return pow2 ? (void *)k_sample<NDIM, float, true> : (void *)k_sample<NDIM, float, false>;
-    else
-        return (void *)k_sample<NDIM, double, false>;
+        if (m.pow2) return (const void *)sample_fn_pow2<NDIM>(m.L, m.priv != 0);
+    return (const void *)k_sample<NDIM, Real>;
 }
 
 template <int NDIM, typename Real>
@@ -2131,14 +2357,14 @@ cudaError_t launch_sample(const SampleArgs<Real> &a, int grid, cudaStream_t s)
 {
     // (sample_occupancy, always called first, sets the shared-memory limit)
     const size_t smem = sample_smem_bytes(NDIM, a.nbins, sizeof(Real) == 8, a.map.priv != 0);
-    if (a.gen == kGenPseudo) {
-        return launch_kernel(k_sample_pseudo<NDIM, Real>, grid, kBlock, smem, s, a);
-    } else if constexpr (sizeof(Real) == 4) {
-        return launch_kernel(a.map.pow2 ? k_sample<NDIM, float, true> : k_sample<NDIM, float, false>, grid, kBlock,
-                             smem, s, a);
-    } else {
-        return launch_kernel(k_sample<NDIM, double, false>, grid, kBlock, smem, s, a);
+    if (a.gen == kGenPseudo) return launch_kernel(k_sample_pseudo<NDIM, Real>, grid, kBlock, smem, s, a);
+    if constexpr (sizeof(Real) == 4) {
+        if (a.map.pow2) {
+            const SampleFn32 f = sample_fn_pow2<NDIM>(a.map.L, a.map.priv != 0);
+            return f ? launch_kernel(f, grid, kBlock, smem, s, a) : cudaErrorInvalidValue;
+        }
     }
+    return launch_kernel(k_sample<NDIM, Real>, grid, kBlock, smem, s, a);
 }
 
 template <int NDIM, typename Real>
@@ -2149,25 +2375,18 @@ cudaError_t sample_occupancy(int nbins, int *blocks_per_sm)
     int optin = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    for (int v = 0; v < 2; ++v) {
-        cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, sample_fn<NDIM, Real>(v == 1));
-        if (e != cudaSuccess) return e;
-        // (the limit, not the launch size: static shared memory counts too)
-        e = cudaFuncSetAttribute(sample_fn<NDIM, Real>(v == 1), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 optin - (int)fa.sharedSizeBytes);
-        if (e != cudaSuccess) return e;
-    }
-    {
-        void *f = (void *)k_sample_pseudo<NDIM, Real>;
+    const void *fn = sample_fn<NDIM, Real>(m);
+    const void *all[2] = {fn, (const void *)k_sample_pseudo<NDIM, Real>};
+    for (const void *f : all) {
+        if (!f) return cudaErrorInvalidValue;
         cudaFuncAttributes fa;
         cudaError_t e = cudaFuncGetAttributes(&fa, f);
         if (e != cudaSuccess) return e;
+        // (the limit, not the launch size: static shared memory counts too)
         e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
         if (e != cudaSuccess) return e;
     }
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, sample_fn<NDIM, Real>(m.pow2 != 0),
-                                                         kBlock, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, kBlock, smem);
 }
 
 template <int NDIM, bool POW2>

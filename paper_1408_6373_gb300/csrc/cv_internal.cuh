@@ -465,19 +465,29 @@ int fp32_range_check(const cv_genz *g, char *msg, size_t len);
 
 // Shared memory of a sampling block: the grid table [ndim][nbins] (FP64:
 // 16-byte {e, w} entries; FP32: 8-byte entries, aligned to 8 nbins bytes),
-// then either one block histogram [ndim][nbins] or, with private
-// histograms, one such copy per warp.
-inline size_t sample_smem_bytes(int ndim, int nbins, bool fp64, bool priv) {
+// then either one block histogram [ndim][nbins] (FP32: and the squares the
+// warps hand to its axes' owners, two rounds of one value per thread) or,
+// with private histograms, one such copy per warp.
+__host__ __device__ constexpr size_t sample_smem_bytes(int ndim, int nbins, bool fp64, bool priv) {
     const size_t entries = (size_t)ndim * nbins * (2 + (priv ? kWarpsPerBlock : 1));
-    return fp64 ? entries * sizeof(double) : entries * sizeof(float) + 8 * (size_t)nbins;
+    return fp64 ? entries * sizeof(double)
+                : entries * sizeof(float) + 8 * (size_t)nbins + (priv ? 0 : 2 * kBlock * sizeof(float));
 }
 
 // Resident 256-thread blocks per SM the FP32 sampling kernels are compiled
 // for (their __launch_bounds__): three up to 8 dimensions, else two.
-inline int min_blocks_f32(int ndim) { return ndim <= 8 ? 3 : 2; }
+constexpr int min_blocks_f32(int ndim) { return ndim <= 8 ? 3 : 2; }
 
 constexpr size_t kSmemPerSM = 228 * 1024;     // shared memory of one SM
 constexpr size_t kSmemBlockReserve = 2048;    // per block: runtime reserve + static arrays
+
+// Every warp's histogram copy fits beside the grid at the occupancy the
+// kernel is compiled for.  (FP64: compiled for one block per SM, but its
+// copies must still leave room for a second.)
+constexpr bool copies_fit(int ndim, int nbins, bool fp64) {
+    return (size_t)(fp64 ? 2 : min_blocks_f32(ndim)) *
+           (sample_smem_bytes(ndim, nbins, fp64, true) + kSmemBlockReserve) <= kSmemPerSM;
+}
 
 #if !defined(__CUDACC_RTC__)
 // Steps in which a warp updates its own f^2 histogram of N bins without
@@ -503,8 +513,7 @@ inline int hist_phases(int N)
 //   the slot is word >> (32 - L) and the fraction's bits sit at mantissa
 //   position: word & mF).  Other N take the generic map.
 //   priv: a warp keeps its own f^2 histogram and updates it with plain loads
-//   and stores, in hist_phases(N) steps.  Used when every warp's copy fits beside
-//   the grid at the occupancy the kernel is compiled for.
+//   and stores, in hist_phases(N) steps, where copies_fit.
 inline MapParams make_map(int N, int ndim, bool fp64)
 {
     MapParams m;
@@ -524,10 +533,7 @@ inline MapParams make_map(int N, int ndim, bool fp64)
         m.li = L - 4;
         m.sA = 29 - L;
     }
-    // (FP64: the kernel is compiled for one block per SM; its copies must
-    // still leave room for a second)
-    const int blocks = fp64 ? 2 : min_blocks_f32(ndim);
-    if ((size_t)blocks * (sample_smem_bytes(ndim, N, fp64, true) + kSmemBlockReserve) <= kSmemPerSM)
+    if (copies_fit(ndim, N, fp64))
         m.priv = hist_phases(N);
     return m;
 }

@@ -141,8 +141,11 @@ std::string specialised_source(const SampleArgs<float> &a, int ndim, bool pow2, 
     std::string s = policy_source(a, ndim, pow2);
     s += "extern \"C\" __global__ void __launch_bounds__(" + std::to_string(kBlock) + ", " +
          std::to_string(min_blocks) + ") cv_jit_sample(const __grid_constant__ cv::SampleArgs<float> A)\n{\n";
-    s += "    cv::sample_pass<" + std::to_string(ndim) + ", float, " + (pow2 ? "true" : "false") +
-         ", cv::JitIntegrand>(A);\n}\n";
+    if (pow2 && !a.map.priv)
+        s += "    cv::sample_pass_owner<" + std::to_string(ndim) + ", cv::JitIntegrand>(A);\n}\n";
+    else
+        s += "    cv::sample_pass<" + std::to_string(ndim) + ", float, " + (pow2 ? "true" : "false") +
+             ", cv::JitIntegrand>(A);\n}\n";
     return s;
 }
 

@@ -120,3 +120,25 @@ def _pass_check(ctx, fams, a, u, edges, start, n, fp64):
     assert np.all(np.abs(S1 - ob.S1) <= 1e-12 * ob.A1)
     assert np.all(np.abs(S2 - ob.S2) <= 1e-12 * ob.S2)
     assert np.all(np.abs(H - ob.H) <= 1e-12 * ob.H.max(axis=1, keepdims=True))
+
+
+@pytest.mark.parametrize("ndim,nbins,flags", [(8, 256, 0), (12, 256, 0), (12, 256, cg.JIT), (23, 128, 0),
+                                              (23, 128, cg.SCRAMBLE), (32, 256, 0)])
+@pytest.mark.parametrize("start,n", [(1, 1), (255, 257), (256, 4096), (1000001, 30011)])
+def test_axes_owned_by_warps(ctx, ndim, nbins, flags, start, n):
+    # (bins and dimensions whose histogram copies do not fit: groups of 256
+    # points, ragged at both ends)
+    rng = np.random.default_rng(ndim)
+    a, u = 0.2 + 0.5 * rng.random((2, ndim)), rng.random((2, ndim))
+    fams = [O.GAUSSIAN, O.C0]
+    edges = np.tile(np.arange(nbins + 1) / nbins, (ndim, 1)) ** 1.1
+    seed = 11
+    p = O.Problem(ndim, fams, a, u, nbins=nbins, bits=23, **(
+        dict(gen=O.SCRAMBLED, seed=seed) if flags & cg.SCRAMBLE else {}))
+    ob = O.sample_bounds(p, edges, start, n)
+    S1 = torch.zeros(2, dtype=torch.float64, device="cuda")
+    S2, H = torch.zeros_like(S1), torch.zeros((ndim, nbins), dtype=torch.float64, device="cuda")
+    ctx.sample(cg.genz(ndim, fams, a, u), nbins, torch.tensor(edges, device="cuda"), start, n, flags, S1, S2, H,
+               seed=seed)
+    ctx.synchronize()
+    check_fp32_pass(S1.cpu().numpy(), S2.cpu().numpy(), H.cpu().numpy(), ob, n)
