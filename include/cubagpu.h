@@ -362,8 +362,9 @@ int cv_vegas_io_bytes(int ndim, int nbins, int64_t *h2d, int64_t *d2h);
  * Execution: in FP32 with Sobol or scrambled points every pass is one
  * batched sampling launch over all its regions (CV_JIT has no effect), the
  * flatness measure computed on the device; FP64 and CV_PSEUDO passes launch
- * once per region and take every decision value on the host.  Memory,
- * allocated per call for max_regions regions: per region ndim (2 nbins + 1)
+ * once per region and take every decision value on the host.  Memory for
+ * max_regions regions, kept on the context from call to call (up to 64 MiB
+ * a buffer, the rest is released when the call returns): per region ndim (2 nbins + 1)
  * doubles of grid and histogram and ~2 KB of descriptors and state on the
  * device, its grid and sums in pinned host memory, and a staging area for
  * up to max(65536, 4 max_regions) tiles.

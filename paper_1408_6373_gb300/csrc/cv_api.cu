@@ -107,6 +107,13 @@ struct cv_ctx {
     size_t parts_cap = 0;
     int parts_G = 0;
     int *pinned = nullptr;  // [0] = 1 (pass_active), [1] = stopped read back
+    // cv_suave's regions (device, pinned host) and its batched form's
+    // descriptors and staging, kept from call to call up to kSuaveKeep bytes
+    // each: allocating and releasing them took 0.3 ms of a 2.3 ms call
+    struct Kept {
+        void *p = nullptr;
+        size_t cap = 0;
+    } suave_dev, suave_host, suave_batch, suave_stage;
     // cv_kernel_timer: event pairs around the sampling launches
     cudaEvent_t tev[2 * CV_TIMER_CAP] = {};
     int timer_on = 0, timer_n = 0;
@@ -199,6 +206,37 @@ extern "C" int cv_create(cv_ctx **out, int device, void *stream)
     return CV_OK;
 }
 
+// Frees what cv_suave keeps on the context beyond `keep` bytes a buffer.
+constexpr size_t kSuaveKeep = 64u << 20;
+static void suave_release(cv_ctx *ctx, size_t keep)
+{
+    for (cv_ctx::Kept *k : {&ctx->suave_dev, &ctx->suave_host, &ctx->suave_batch, &ctx->suave_stage}) {
+        if (!k->p || (keep && k->cap <= keep)) continue;
+        if (k == &ctx->suave_host || k == &ctx->suave_stage) cudaFreeHost(k->p);
+        else cudaFree(k->p);
+        *k = {};
+    }
+}
+
+// A kept buffer of at least `bytes` (its contents are not kept); false when
+// it cannot be had.
+static bool suave_take(cv_ctx::Kept *k, size_t bytes, bool host)
+{
+    if (k->p && k->cap >= bytes) return true;
+    if (k->p) {
+        if (host) cudaFreeHost(k->p);
+        else cudaFree(k->p);
+    }
+    *k = {};
+    if ((host ? cudaMallocHost(&k->p, bytes) : cudaMalloc(&k->p, bytes)) != cudaSuccess) {
+        cudaGetLastError();
+        *k = {};
+        return false;
+    }
+    k->cap = bytes;
+    return true;
+}
+
 extern "C" void cv_destroy(cv_ctx *ctx)
 {
     if (!ctx) return;
@@ -221,6 +259,7 @@ extern "C" void cv_destroy(cv_ctx *ctx)
     if (ctx->mat_mem) cudaFree(ctx->mat_mem);
     if (ctx->vegas_mem) cudaFree(ctx->vegas_mem);
     if (ctx->parts_mem) cudaFree(ctx->parts_mem);
+    suave_release(ctx, 0);
     if (ctx->pinned) cudaFreeHost(ctx->pinned);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
@@ -3120,6 +3159,23 @@ struct SuaveMem {
     double *dh_edges = nullptr, *dh_S = nullptr, *dh_fluct = nullptr;  // device addresses of the mirrors
 };
 
+// Region k's descriptor: `proto` with region k's state, grid (ge doubles) and
+// histogram (gh doubles) for region 0's.
+__global__ void k_suave_items(const __grid_constant__ BatchItem proto, BatchItem *items, int ge, int gh)
+{
+    wait_for_previous();
+    const size_t k = blockIdx.x;
+    const int *src = reinterpret_cast<const int *>(&proto.a);
+    int *dst = reinterpret_cast<int *>(&items[k].a);
+    for (int i = threadIdx.x; i < (int)(sizeof(proto.a) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
+    if (threadIdx.x == 0) {
+        items[k].st = proto.st + k;
+        items[k].edges = proto.edges + k * ge;
+        items[k].H = proto.H + k * gh;
+        items[k].ew32 = nullptr;
+    }
+}
+
 __global__ void k_suave_prep(const SuaveEntry *E, const BatchItem *items, const double *dh_edges, int ndim,
                              int N, long long nnew, int *counter)
 {
@@ -3163,9 +3219,16 @@ __global__ void k_suave_gather(const SuaveEntry *E, const BatchItem *items, doub
         const double *e = it.edges + (size_t)d * (N + 1);
         const double mean = (e[N] - e[0]) / N;
         double acc = 0.0;
-        for (int k = lane; k < N; k += 32) acc += pow(fabs(log((e[k + 1] - e[k]) / mean)), flatness);
+        // (the default flatness of 2 as a square and a square root, correctly
+        // rounded; two calls of pow are most of this kernel's time otherwise,
+        // 16 us a launch)
+        const bool two = flatness == 2.0;
+        for (int k = lane; k < N; k += 32) {
+            const double x = log((e[k + 1] - e[k]) / mean);
+            acc += two ? x * x : pow(fabs(x), flatness);
+        }
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) dh_fluct[(size_t)CV_MAX_DIM * r + d] = pow(acc / N, 1.0 / flatness);
+        if (lane == 0) dh_fluct[(size_t)CV_MAX_DIM * r + d] = two ? sqrt(acc / N) : pow(acc / N, 1.0 / flatness);
     }
 }
 
@@ -3435,7 +3498,7 @@ int suave_run(cv_ctx *ctx, const cv_genz *g, int N, int flags, uint64_t seed, do
 // points, a region's pass within the tiles' int range and a grid that fits
 // the batched kernel's shared memory.  Otherwise m stays per-region.
 int suave_batched_setup(cv_ctx *ctx, const cv_genz *g, int N, int flags, uint64_t seed, long long nnew,
-                        int max_regions, SuaveMem &m, void **bmem, void **hstage)
+                        int max_regions, SuaveMem &m)
 {
     const int ndim = g->ndim;
     if ((flags & (CV_FP64 | CV_PSEUDO)) || nnew > (1LL << 31)) return CV_OK;
@@ -3450,17 +3513,11 @@ int suave_batched_setup(cv_ctx *ctx, const cv_genz *g, int N, int flags, uint64_
     const size_t sz_state = align16((size_t)max_regions * sizeof(DevState));
     const size_t sz_stage = align16((size_t)max_regions * sizeof(SuaveEntry)) + (size_t)tile_cap * sizeof(Tile) +
                             (size_t)max_regions * ndim * sizeof(int2) + 64;
-    char *d = nullptr;
-    if (cudaMalloc((void **)&d, sz_items + sz_state + sz_stage + 16) != cudaSuccess) {
-        cudaGetLastError();
+    if (!suave_take(&ctx->suave_batch, sz_items + sz_state + sz_stage + 16, false))
         return fail_msg(ctx, CV_ENOMEM, "device allocation of the batched regions failed");
-    }
-    *bmem = d;
-    if (cudaMallocHost(hstage, sz_stage) != cudaSuccess) {
-        cudaGetLastError();
-        *hstage = nullptr;
+    if (!suave_take(&ctx->suave_stage, sz_stage, true))
         return fail_msg(ctx, CV_ENOMEM, "pinned staging allocation failed");
-    }
+    char *const d = static_cast<char *>(ctx->suave_batch.p);
     // (the mirrors are one mapped pinned allocation starting at h_edges)
     CV_CUDA(ctx, cudaHostGetDevicePointer((void **)&m.dh_edges, m.h_edges, 0));
     m.dh_S = m.dh_edges + (m.h_S - m.h_edges);
@@ -3469,12 +3526,13 @@ int suave_batched_setup(cv_ctx *ctx, const cv_genz *g, int N, int flags, uint64_
     DevState *st = m.d_state = reinterpret_cast<DevState *>(d + sz_items);
     m.d_stage = d + sz_items + sz_state;
     m.d_counter = reinterpret_cast<int *>(m.d_stage + sz_stage);
-    m.h_stage = static_cast<char *>(*hstage);
+    m.h_stage = static_cast<char *>(ctx->suave_stage.p);
     m.tile_cap = tile_cap;
     m.grid = ctx->sms * occ;
     m.pow2 = pow2;
     const size_t ge = (size_t)ndim * (N + 1), gh = (size_t)ndim * N;
-    std::vector<BatchItem> items((size_t)max_regions);
+    // (all regions' descriptors are one, but for their places: written on the
+    // device, not copied)
     BatchItem proto;
     memset(&proto, 0, sizeof(proto));
     fill_params<float>(g, &proto.a.g);
@@ -3483,16 +3541,11 @@ int suave_batched_setup(cv_ctx *ctx, const cv_genz *g, int N, int flags, uint64_
     proto.a.map = make_map(N, ndim, false);
     proto.a.map.priv = hist_phases(N);  // (every warp has its own histogram)
     set_generator(&proto.a, ndim, flags, seed);
-    for (int k = 0; k < max_regions; ++k) {
-        items[(size_t)k] = proto;
-        items[(size_t)k].st = st + k;
-        items[(size_t)k].edges = m.edges + ge * k;
-        items[(size_t)k].H = m.H + gh * k;
-    }
+    proto.st = st;
+    proto.edges = m.edges;
+    proto.H = m.H;
     CV_CUDA(ctx, cudaMemsetAsync(st, 0, sz_state, ctx->stream));
-    CV_CUDA(ctx, cudaMemcpyAsync(m.d_items, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice,
-                                 ctx->stream));
-    CV_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    CV_CUDA(ctx, launch_kernel(k_suave_items, max_regions, 128, 0, ctx->stream, proto, m.d_items, (int)ge, (int)gh));
     m.batched = true;
     return CV_OK;
 }
@@ -3522,34 +3575,25 @@ extern "C" int cv_suave(cv_ctx *ctx, const cv_genz *g, int nbins, int flags, uin
     const size_t ge = (size_t)ndim * (nbins + 1), gh = (size_t)ndim * nbins, gs = 2 * CV_MAX_COMP;
     SuaveMem m;
     const size_t bytes = sizeof(double) * (ge + gh + gs) * (size_t)max_regions;
-    void *mem = nullptr;
-    if (cudaMalloc(&mem, bytes) != cudaSuccess) {
-        cudaGetLastError();
+    if (!suave_take(&ctx->suave_dev, bytes, false))
         return fail_msg(ctx, CV_ENOMEM, "device allocation for %d regions failed", max_regions);
-    }
-    m.edges = (double *)mem;
+    m.edges = (double *)ctx->suave_dev.p;
     m.H = m.edges + ge * (size_t)max_regions;
     m.S = m.H + gh * (size_t)max_regions;
-    void *hmem = nullptr;
-    if (cudaMallocHost(&hmem, sizeof(double) * (ge + gs + CV_MAX_DIM) * (size_t)max_regions) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(mem);
+    if (!suave_take(&ctx->suave_host, sizeof(double) * (ge + gs + CV_MAX_DIM) * (size_t)max_regions, true)) {
+        suave_release(ctx, kSuaveKeep);
         return fail_msg(ctx, CV_ENOMEM, "pinned host allocation for %d regions failed", max_regions);
     }
-    m.h_edges = (double *)hmem;
+    m.h_edges = (double *)ctx->suave_host.p;
     m.h_S = m.h_edges + ge * (size_t)max_regions;
     m.h_fluct = m.h_S + gs * (size_t)max_regions;
-    void *bmem = nullptr, *hstage = nullptr;
-    rc = suave_batched_setup(ctx, g, nbins, flags, seed, nnew, max_regions, m, &bmem, &hstage);
+    rc = suave_batched_setup(ctx, g, nbins, flags, seed, nnew, max_regions, m);
     if (rc == CV_OK) rc = (flags & CV_FP64)
         ? suave_run<double>(ctx, g, nbins, flags, seed, epsrel, epsabs, mineval, maxeval, nnew, flatness, width,
                             max_regions, m, nregions, neval, fail, integral, error, boxes)
         : suave_run<float>(ctx, g, nbins, flags, seed, epsrel, epsabs, mineval, maxeval, nnew, flatness, width,
                            max_regions, m, nregions, neval, fail, integral, error, boxes);
     cudaStreamSynchronize(ctx->stream);
-    cudaFree(mem);
-    cudaFreeHost(hmem);
-    if (bmem) cudaFree(bmem);
-    if (hstage) cudaFreeHost(hstage);
+    suave_release(ctx, kSuaveKeep);
     return rc;
 }
