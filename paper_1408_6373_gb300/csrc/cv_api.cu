@@ -2945,10 +2945,9 @@ static int vegas_cb_run(cv_ctx *ctx, int ndim, int ncomp, cv_integrand_dev cb, v
     if (rc) return rc;
     pin[0] = 1;
     int aborted = 0;
-    // (the dimension-major FP32 kernels for N = 2^L flag the refinement
-    // themselves: their accumulate pass sets pass_active from the stop flag)
-    const bool lean = fp32 && a.map.pow2 && !aos && a.gen != kGenPseudo && a.map.priv;
-    if (lean) a.st = st;
+    // (the FP32 accumulate kernels for N = 2^L flag the refinement
+    // themselves: they set pass_active from the stop flag)
+    const bool lean = fp32 && a.map.pow2 && a.gen != kGenPseudo && a.map.priv;
     // the stop flag through host-mapped memory (no copy per iteration),
     // where the pinned buffer has a device address
     int *host_stop = nullptr;
@@ -3013,6 +3012,7 @@ static int vegas_cb_run(cv_ctx *ctx, int ndim, int ncomp, cv_integrand_dev cb, v
             b.n = m;
             parts_args(&pp, 0, &b.part_S, &b.part_H, &b.part_ticket);
             b.part_G = pp.G_cap;
+            if (lean) b.st = st;
             if (one_tile) b.part_ticket = nullptr;  // (the combination adds the sums)
             e = dispatch_matpass<Real>(ndim, true, b, mat_grid(ctx, occ, m), s, &grid_used);
             if (e == cudaSuccess && !one_tile)

@@ -783,6 +783,26 @@ __device__ __forceinline__ void sample_block(const SampleArgs<float> &A, const S
             float x[NDIM];
 #pragma unroll
             for (int d = 0; d < NDIM; ++d) x[d] = z[d] + 0.5f;
+            if (!EDGE && A.aos && hmode != kHistBlock && N >= 64) {
+                // point-major: the block's 32 NDIM values are one run in x,
+                // put in order in the space of this warp's histogram (unused
+                // here; an odd stride keeps the lanes' writes apart) and
+                // stored 32 at a time.  (Stored as they come, every store
+                // touches all of the run's lines: 17 us for 1e6 points of 5
+                // dimensions, 9 us so.)
+                constexpr int S = NDIM | 1;
+                __syncwarp();
+#pragma unroll
+                for (int d = 0; d < NDIM; ++d) sm.h[lane * S + d] = x[d];
+                __syncwarp();
+                float *xp = A.x + (long long)(q * 32ull - start) * NDIM + lane;
+#pragma unroll
+                for (int k = 0; k < NDIM; ++k) {
+                    const int e = k * 32 + lane, pt = e / NDIM;
+                    xp[k * 32] = sm.h[pt * S + (e - pt * NDIM)];
+                }
+                return;
+            }
             store_point<NDIM, float>(A, (long long)(q * 32ull + (unsigned long long)lane - start), x);
         }
         return;
@@ -1999,7 +2019,9 @@ __device__ __forceinline__ int group_step_word(int kk)
 // ring (each lane copies and later reads only its own words; points outside
 // copy zeros).  Plain FP32 partial sums over runs of kRun blocks are folded
 // into the per-thread Kahan sums after each run (as in the fused pass).
-template <int NDIM, int L, bool EDGE>
+// AOS: value c of point j at f[j ncomp + c] instead of f[c ld + j] (1e6
+// points, 5 dimensions, 2 components: 14.1 us, the general pass 18.7).
+template <int NDIM, int L, bool EDGE, bool AOS>
 __device__ __forceinline__ void mat_accum_chunk(const SampleArgs<float> &A, const Smem<float> &sm,
                                                 unsigned long long q0, int nk, int lane, unsigned ring,
                                                 int ncomp, Acc<float> (&s1)[CV_MAX_COMP],
@@ -2021,14 +2043,22 @@ __device__ __forceinline__ void mat_accum_chunk(const SampleArgs<float> &A, cons
         static_assert(kMatAhead == kMatGroup, "one ring stage per block of a group");
         // this lane's values of the group's blocks: component c of block
         // k0 + kk at pv[c] + 32 kk (the pointers advance by a group)
+        // (point-major: the point's values from one pointer, which moves on
+        // with every block requested)
         const float *pv[CV_MAX_COMP];
 #pragma unroll
-        for (int c = 0; c < CV_MAX_COMP; ++c) pv[c] = A.f + j0 + c * ld;
-#pragma unroll
-        for (int kk = 0; kk < kMatGroup; ++kk) {
+        for (int c = 0; c < CV_MAX_COMP; ++c) pv[c] = A.f + (AOS ? j0 * ncomp : j0 + c * ld);
+        const int next = 32 * ncomp;
+        auto ask = [&](int kk) {
 #pragma unroll
             for (int c = 0; c < CV_MAX_COMP; ++c)
-                if (c < ncomp) cp_async4_full(ring + kk * kStage + (unsigned)(c * 128), pv[c] + 32 * kk);
+                if (c < ncomp)
+                    cp_async4_full(ring + kk * kStage + (unsigned)(c * 128), AOS ? pv[0] + c : pv[c] + 32 * kk);
+            if constexpr (AOS) pv[0] += next;
+        };
+#pragma unroll
+        for (int kk = 0; kk < kMatGroup; ++kk) {
+            ask(kk);
             cp_async_commit();
         }
         // groups of kMatGroup blocks from multiples of kMatGroup: the step
@@ -2039,8 +2069,10 @@ __device__ __forceinline__ void mat_accum_chunk(const SampleArgs<float> &A, cons
         // the stage block kk has just left
         for (int k0 = 0; k0 < nk; k0 += kMatGroup) {
             const bool more = k0 + kMatGroup < nk;
+            if constexpr (!AOS) {
 #pragma unroll
-            for (int c = 0; c < CV_MAX_COMP; ++c) pv[c] += 32 * kMatGroup;
+                for (int c = 0; c < CV_MAX_COMP; ++c) pv[c] += 32 * kMatGroup;
+            }
 #pragma unroll
             for (int kk = 0; kk < kMatGroup; ++kk) {
                 cp_async_wait<kMatAhead - 1>();  // (block k0 + kk's copies have landed)
@@ -2055,11 +2087,7 @@ __device__ __forceinline__ void mat_accum_chunk(const SampleArgs<float> &A, cons
                 } else if (more) {
                     sobol_step<NDIM, unsigned>(X, q0 + (unsigned long long)(k0 + kk), P::li);
                 }
-                if (more) {
-#pragma unroll
-                    for (int c = 0; c < CV_MAX_COMP; ++c)
-                        if (c < ncomp) cp_async4_full(ring + kk * kStage + (unsigned)(c * 128), pv[c] + 32 * kk);
-                }
+                if (more) ask(kk);
                 cp_async_commit();
             }
             if (((k0 + kMatGroup) % (int)kRun) == 0) mat_fold(Pt, ncomp, s1, s2);
@@ -2069,14 +2097,15 @@ __device__ __forceinline__ void mat_accum_chunk(const SampleArgs<float> &A, cons
         const int klo = j0 >= 0 ? 0 : (int)((31 - j0) / 32);
         const long long r = A.n - j0;
         const int khi = r <= 0 ? 0 : (int)min((long long)nk, (r + 31) / 32);
-        const float *pf = A.f + j0;  // (dereferenced at valid k only)
+        const long long sj = AOS ? ncomp : 1, sc = AOS ? 1 : ld;
+        const float *pf = A.f + j0 * sj;  // (dereferenced at valid k only)
         auto request = [&](int k) {
             const unsigned stage = ring + (unsigned)((k & (kMatAhead - 1)) * kStage);
             const bool v = k >= klo && k < khi;
-            const float *src = v ? pf + 32 * k : A.f;
+            const float *src = v ? pf + 32 * k * sj : A.f;
 #pragma unroll
             for (int c = 0; c < CV_MAX_COMP; ++c)
-                if (c < ncomp) cp_async4(stage + (unsigned)(c * 128), src + c * ld, v ? 4u : 0u);
+                if (c < ncomp) cp_async4(stage + (unsigned)(c * 128), src + c * sc, v ? 4u : 0u);
             cp_async_commit();
         };
         auto block = [&](int k) {
@@ -2107,7 +2136,7 @@ __device__ __forceinline__ void mat_accum_chunk(const SampleArgs<float> &A, cons
 // bits), so each warp's f^2 histogram copy takes plain updates (the 32
 // lanes' bins are distinct); sums and histogram as the fused pass.  N = 2^L
 // at compile time.
-template <int NDIM, int L>
+template <int NDIM, int L, bool AOS>
 __global__ void __launch_bounds__(kBlock, kMatAccumBlocks)
 k_mat_accum(const __grid_constant__ SampleArgs<float> A)
 {
@@ -2168,9 +2197,9 @@ k_mat_accum(const __grid_constant__ SampleArgs<float> A)
         const unsigned long long q0 = qa + ch * per;
         const int nk = (int)min(per, qb - q0);
         if ((unsigned long long)nk == per && q0 * 32ull >= start && (q0 + per) * 32ull <= start + (unsigned long long)n)
-            mat_accum_chunk<NDIM, L, false>(A, sm, q0, nk, lane, ring, ncomp, s1, s2);
+            mat_accum_chunk<NDIM, L, false, AOS>(A, sm, q0, nk, lane, ring, ncomp, s1, s2);
         else
-            mat_accum_chunk<NDIM, L, true>(A, sm, q0, nk, lane, ring, ncomp, s1, s2);
+            mat_accum_chunk<NDIM, L, true, AOS>(A, sm, q0, nk, lane, ring, ncomp, s1, s2);
     }
     const int N = P::N;
 
@@ -2432,13 +2461,14 @@ static cudaError_t launch_mat_lean(const SampleArgs<float> &a, int grid, cudaStr
     // table, the warps' value rings)
     const size_t smem = (size_t)(1 + kWarpsPerBlock) * NDIM * P::N * 4 + 8 * (size_t)P::N +
                         (size_t)kWarpsPerBlock * kMatAhead * CV_MAX_COMP * 32 * 4;
-    cudaError_t e = cudaFuncSetAttribute(k_mat_accum<NDIM, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = a.aos ? k_mat_accum<NDIM, L, true> : k_mat_accum<NDIM, L, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // (at most one wave of this kernel's own residency)
-    static int occ = 0;
+    static int occ = 0;  // (both layouts: compiled for kMatAccumBlocks)
     int dev = 0, sms = 0;
     if (!occ) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mat_accum<NDIM, L>, kBlock, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kBlock, smem);
         if (e != cudaSuccess) return e;
         if (occ < 1) occ = 1;
     }
@@ -2448,16 +2478,17 @@ static cudaError_t launch_mat_lean(const SampleArgs<float> &a, int grid, cudaStr
     if (grid > sms * occ) grid = sms * occ;
     if (a.part_S && grid > a.part_G) return cudaErrorInvalidValue;  // (partial rows for every block)
     *grid_used = grid;
-    return launch_kernel(k_mat_accum<NDIM, L>, grid, kBlock, smem, s, a);
+    return launch_kernel(kernel, grid, kBlock, smem, s, a);
 }
 
 template <int NDIM, typename Real, bool POW2, int MODE>
 static cudaError_t launch_matpass_v(const SampleArgs<Real> &a, int grid, cudaStream_t s, int *grid_used)
 {
     if constexpr (sizeof(Real) == 4 && POW2) {
-        // the common case's own kernels (dimension-major, Sobol points; the
-        // accumulate pass needs the warps' histogram copies to fit)
-        if (!a.aos && a.gen != kGenPseudo && (MODE == 1 || a.map.priv)) {
+        // the common case's own kernels (Sobol points; the store pass
+        // dimension-major, the accumulate pass where the warps' histogram
+        // copies fit)
+        if (a.gen != kGenPseudo && (MODE == 1 ? !a.aos : a.map.priv != 0)) {
             switch (a.map.L) {
             case 5: return launch_mat_lean<NDIM, 5, MODE>(a, grid, s, grid_used);
             case 6: return launch_mat_lean<NDIM, 6, MODE>(a, grid, s, grid_used);
