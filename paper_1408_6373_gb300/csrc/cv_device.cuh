@@ -1136,8 +1136,8 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
     const int ncomp = A.g.ncomp;
     // warp copies of the histogram for Sobol points when they fit
     // (FP32 power-of-two passes whose copies do not fit: sample_pass_owner)
-    const bool priv = I::kGen != 2 && (sizeof(Real) == 4 ? (POW2 && I::kMode == 0) || I::priv(A.map) : A.map.priv != 0);
-    const int hmode = !priv ? kHistBlock : (sizeof(Real) == 4 && POW2 ? kHistWarpPlain : kHistWarpPhased);
+    const bool priv = I::kGen != 2 && (sizeof(Real) == 4 ? POW2 && (I::kMode == 0 || I::priv(A.map)) : A.map.priv != 0);
+    const int hmode = !priv ? kHistBlock : sizeof(Real) == 4 ? kHistWarpPlain : kHistWarpPhased;
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem<Real> sm;

@@ -481,12 +481,13 @@ constexpr int min_blocks_f32(int ndim) { return ndim <= 8 ? 3 : 2; }
 constexpr size_t kSmemPerSM = 228 * 1024;     // shared memory of one SM
 constexpr size_t kSmemBlockReserve = 2048;    // per block: runtime reserve + static arrays
 
-// Every warp's histogram copy fits beside the grid at the occupancy the
-// kernel is compiled for.  (FP64: compiled for one block per SM, but its
-// copies must still leave room for a second.)
+// Every warp's histogram copy fits beside the grid with two blocks on an SM
+// (FP32 blocks of up to 8 dimensions are compiled for three, but 8
+// dimensions x 256 bins run faster with two blocks' own copies, 86 us a pass
+// of 1e7 points, than with three blocks whose warps own rows of one copy, 130
+// us, or share it with atomics, 110 us).
 constexpr bool copies_fit(int ndim, int nbins, bool fp64) {
-    return (size_t)(fp64 ? 2 : min_blocks_f32(ndim)) *
-           (sample_smem_bytes(ndim, nbins, fp64, true) + kSmemBlockReserve) <= kSmemPerSM;
+    return 2 * (sample_smem_bytes(ndim, nbins, fp64, true) + kSmemBlockReserve) <= kSmemPerSM;
 }
 
 #if !defined(__CUDACC_RTC__)
@@ -496,9 +497,9 @@ constexpr bool copies_fit(int ndim, int nbins, bool fp64) {
 // strata (N < 32), so the lanes whose strata agree mod 32/N hit distinct
 // bins; from 32 bins on all lanes do.  Other N: two points m strata apart are
 // more than (m - 1)/32 apart, so for a power of two m with (m - 1)/32 >= 1/N
-// the lanes whose strata agree mod m hit distinct bins.  (An FP32 or FP64 add
-// on shared memory is a compare-and-swap loop on this GPU, and one copy for
-// the whole block makes the warps collide.)
+// the lanes whose strata agree mod m hit distinct bins.  (An add on shared
+// memory is a compare-and-swap loop on this GPU; what the steps gain over it,
+// and where they do not: make_map.)
 inline int hist_phases(int N)
 {
     if ((N & (N - 1)) == 0) return N >= 32 ? 1 : 32 / N;
@@ -533,8 +534,12 @@ inline MapParams make_map(int N, int ndim, bool fp64)
         m.li = L - 4;
         m.sA = 29 - L;
     }
-    if (copies_fit(ndim, N, fp64))
-        m.priv = hist_phases(N);
+    // (a single FP32 pass with other bin counts shares one copy per block:
+    // two steps of predicated loads and stores cost it more than the
+    // shared-memory atomics do, 8 dimensions x 50 bins, 1e7 points 155 against
+    // 128 us; FP64 takes 110 against 120 us for 3 dimensions x 50 bins, 1e6
+    // points, and the batched kernel's warps 580 against 652 us for 6)
+    if ((fp64 || m.pow2) && copies_fit(ndim, N, fp64)) m.priv = hist_phases(N);
     return m;
 }
 
