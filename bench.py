@@ -720,7 +720,7 @@ def run_ours(args):
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "kernel": f"sampling kernel, ndim {p.ndim}, FP32, specialised at run time"
-                               if jit_compiled else f"k_sample<{p.ndim},float>",
+                               if jit_compiled else f"k_sample_pow2<{p.ndim},{p.nbins.bit_length() - 1}>",
                      "kernel_ms": k_ms, "kernel_ms_generic": k_ms_generic,
                      "kernel_ms_in_vegas_runs": k_ms_in_run, "launches_in_vegas_runs": len(in_run),
                      "jit": {"available": jit_available, "compiled": jit_compiled},
