@@ -505,10 +505,8 @@ void cv_integral_destroy(cv_integral *I);
  * forces one size), and each tile leaves its sums and histogram as
  * partial rows that the refinement and combination add in tile order (no
  * floating-point atomics), so an integral's result is the same alone, in
- * any batch and on every run, bit for bit, for the same tile cap and split
- * (with nbins other than 2^L >= 32 a warp's histogram copy takes shared-
- * memory atomics, whose order within a tile the hardware picks).  It
- * agrees with cv_vegas within the FP32 tolerance (the single-integral
+ * any batch and on every run, bit for bit, for the same tile cap and split.
+ * It agrees with cv_vegas within the FP32 tolerance (the single-integral
  * kernel groups points differently). */
 typedef struct cv_batch cv_batch;
 int cv_batch_create(cv_ctx *ctx, int count, const cv_spec *specs, cv_batch **out);
@@ -550,8 +548,7 @@ int cv_batch_vegas(cv_ctx *ctx, int count, const cv_spec *specs, cv_result *out)
  * next round boundary).  A request whose goal or budget is reached leaves
  * at once and frees its slot and memory.  Each request's result is the
  * same alone and in any mix of requests, bit for bit (see cv_batch_create
- * for the tiling rule, the partial rows, the ndim * nbins limit and the
- * bin counts this holds for).
+ * for the tiling rule, the partial rows and the ndim * nbins limit).
  * The analogue of the paper's spinning cores (Sect. 3.2.3): the worker and
  * its device state persist between integrations until cv_server_stop. */
 typedef struct {

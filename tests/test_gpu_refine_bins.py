@@ -1,7 +1,7 @@
 """The refinement's integer arithmetic and the histograms of every bin count.
 
-- cv_refine against the same refinement in extended precision (128-bit long
-  double on the GPU machine's Arm cores), within 1e-14: the weights carry 2^-55 of
+- cv_refine against the same refinement in numpy's extended precision (long
+  double), within 1e-14: the weights carry 2^-55 of
   their scale, their sums are exact, and the logarithm and power behind them
   are good to 2^-49, so an edge is off by less than that over the smallest
   share of a bin these histograms give an edge (~0.1).
