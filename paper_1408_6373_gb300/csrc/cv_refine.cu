@@ -13,6 +13,7 @@
 // probability P((m-1)/2, chi^2/2) uses the regularized incomplete gamma
 // function (series for x < a+1, Legendre continued fraction otherwise).
 #include "cv_internal.cuh"
+#include "cv_rows.h"
 
 namespace cv {
 
@@ -343,8 +344,11 @@ struct Sum64 {
 
 // Space of the row groups' sums of a CTA of 512 threads, and of one of 256
 // (then the bins' prefix sums, weights and reciprocals).
-constexpr int kGroupBytes = 2304 * 8, kGroupBytesBatch = 1152 * 8;
+// (row_entries covers 512 threads and the fewer of a pass of few rows alike:
+// fewer threads form fewer groups.)
+constexpr int kGroupBytes = row_entries(512, CV_MAX_BINS) * 8, kGroupBytesBatch = row_entries(256, CV_MAX_BINS) * 8;
 static_assert(kGroupBytesBatch >= (3 * CV_MAX_BINS + 1) * 8, "the bins' 64-bit values fit");
+static_assert(kGroupBytes % 16 == 0 && kGroupBytesBatch % 16 == 0, "");
 
 // The sums over the G partial rows of one axis (first row P, row stride nh)
 // into sH, by all the CTA's threads: R groups of threads take every R-th
@@ -363,18 +367,9 @@ __device__ __forceinline__ void sum_rows(const CombineArgs *pa, int d, int N, un
     E *grp = reinterpret_cast<E *>(raw);
     const int G = pa->part_G;
     const size_t nh = (size_t)pa->part_nh;
-    // Threads per bin (2^lT) and a group stride that keeps their reads apart
-    // in the banks.  FP64 additions cost 16 cycles of the SM per warp, so
-    // FP64 rows take at most eight groups.  (c32 = ceil(2^32 / N): quotients
-    // of values below 2^16 by N.)
-    const int lT = min(sizeof(T) == 8 ? 3 : 5, 31 - __clz((int)__umulhi(blockDim.x, c32)));
-    const int T2 = 1 << lT;
-    const int stride = ((N + 15) & ~15) + (lT >= 4 ? 1 : 16 >> lT);
-    const int cols = N / V;
-    int R = min((int)__umulhi(blockDim.x * V, c32), G);
-    if (sizeof(T) == 8) R = min(R, 8);
-    if (N < 64) R = min(R, GROUP / (int)(sizeof(E) * stride));
-    const int t = threadIdx.x, r = (int)__umulhi((unsigned)t * V, c32), q = t - r * cols;
+    const RowGroups rg = row_groups((int)blockDim.x, N, c32, sizeof(T) == 8, G, GROUP / (int)sizeof(E));
+    const int lT = rg.lT, T2 = 1 << lT, stride = rg.stride, R = rg.R, cols = N / V;
+    const int t = threadIdx.x, r = row_quotient(t * V, c32), q = t - r * cols;
     if (r < R) {
         S<V> s;
         s.clear();
@@ -474,16 +469,17 @@ __device__ void refine_axis(int d, int N, double *H, double *edges, int zero_his
             lc[i] = g_log.c[at];
         }
     }
-    const unsigned q32 = 0xffffffffu / (unsigned)N, c32 = q32 + 1u;  // (c32 = ceil(2^32 / N))
+    const unsigned c32 = row_reciprocal(N), q32 = c32 - 1u;
     const bool f32 = pa && pa->part_H && pa->part_f32;
     if (f32) {
         float2 *sums = reinterpret_cast<float2 *>(sH_raw);
-        if (N % 4 == 0) sum_rows<GROUP, float, Sum32, float2, 4>(pa, d, N, c32, grp_raw, sums, map);
-        else if (N % 2 == 0) sum_rows<GROUP, float, Sum32, float2, 2>(pa, d, N, c32, grp_raw, sums, map);
+        const int V = row_vector(N, false);
+        if (V == 4) sum_rows<GROUP, float, Sum32, float2, 4>(pa, d, N, c32, grp_raw, sums, map);
+        else if (V == 2) sum_rows<GROUP, float, Sum32, float2, 2>(pa, d, N, c32, grp_raw, sums, map);
         else sum_rows<GROUP, float, Sum32, float2, 1>(pa, d, N, c32, grp_raw, sums, map);
     } else if (pa && pa->part_H) {
         double *sums = reinterpret_cast<double *>(sH_raw);
-        if (N % 2 == 0) sum_rows<GROUP, double, Sum64, double, 2>(pa, d, N, c32, grp_raw, sums, map);
+        if (row_vector(N, true) == 2) sum_rows<GROUP, double, Sum64, double, 2>(pa, d, N, c32, grp_raw, sums, map);
         else sum_rows<GROUP, double, Sum64, double, 1>(pa, d, N, c32, grp_raw, sums, map);
     } else {
         if (k < N) reinterpret_cast<double *>(sH_raw)[k] = Hd[k];
