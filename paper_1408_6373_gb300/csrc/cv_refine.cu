@@ -277,8 +277,7 @@ __device__ __forceinline__ void load_vec(const T *p, T (&v)[V])
 }
 
 // A running sum of V neighbouring values: FP32 with Kahan's compensation
-// (value s - c, kept as s and n = -c), two values per packed instruction;
-// FP64 plain.
+// (row_add, two values per packed instruction); FP64 plain.
 template <int V>
 struct Sum32 {
     float s[V], n[V];
@@ -290,10 +289,7 @@ struct Sum32 {
     __device__ __forceinline__ void add(const float (&v)[V])
     {
         if constexpr (V == 1) {
-            const float y = v[0] + n[0];
-            const float u = s[0] + y;
-            n[0] = y - (u - s[0]);
-            s[0] = u;
+            row_add(s[0], n[0], v[0]);
         } else {
             const float2 m1 = make_float2(-1.0f, -1.0f);
 #pragma unroll
@@ -314,11 +310,7 @@ struct Sum32 {
 // One value's sum in a group, (s, n) or the FP64 sum.
 __device__ __forceinline__ void group_add(float2 &a, const float2 &b)
 {
-    Sum32<1> t{{a.x}, {a.y}};
-    const float x[1] = {b.x}, y[1] = {b.y};
-    t.add(x);
-    t.add(y);
-    a = make_float2(t.s[0], t.n[0]);
+    pair_add(a.x, a.y, b.x, b.y);
 }
 __device__ __forceinline__ void group_add(double &a, const double &b) { a += b; }
 __device__ __forceinline__ float2 group_peer(const float2 &a, int o)

@@ -1,6 +1,7 @@
 // cv_rows.h -- how a refinement CTA adds the partial rows of an axis: the
-// split of its threads and the space it needs.  Plain C++ besides the CUDA
-// qualifiers, so that the host can evaluate it for every bin count.
+// split of its threads, the space it needs and the compensated additions.
+// Plain C++ besides the CUDA qualifiers, so that the host can evaluate it for
+// every bin count.
 #pragma once
 
 #if defined(__CUDACC__)
@@ -54,6 +55,29 @@ CV_ROWS_FN int row_entries(int threads, int bins)
             if (g.R * g.stride > most) most = g.R * g.stride;
         }
     return most;
+}
+
+// A running binary32 sum with Kahan's compensation: value s + n.  The rounding
+// of v + n is dropped, 2^-25 of a row each: 1e-9 of the sum of 456 rows (rms).
+CV_ROWS_FN void row_add(float &s, float &n, float v)
+{
+    const float y = v + n;
+    const float u = s + y;
+    n = y - (u - s);
+    s = u;
+}
+
+// (s + n) += (bs + bn), two sums of like size: the rounding of s + bs is
+// taken exactly (Knuth's TwoSum) and joins the low parts.  (Adding bs and
+// then bn as rows loses half an ulp of the sum at every level of the tree:
+// 456 rows 1.4e-8 off, 152 rows 1.9e-8, 32 rows 1.9e-8; so 0.9e-9, 1.5e-9
+// and 2.6e-9, the rows' own.)
+CV_ROWS_FN void pair_add(float &s, float &n, float bs, float bn)
+{
+    const float u = s + bs;
+    const float t = u - s;
+    n = ((s - (u - t)) + (bs - t)) + (n + bn);
+    s = u;
 }
 
 }  // namespace cv
