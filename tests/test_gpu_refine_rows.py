@@ -60,6 +60,7 @@ def test_one_integral(ctx, N, n, fp64):
         n = 300000
     g, flags = _genz(N), cg.FP64 if fp64 else 0
     I = ctx.integral(cg.spec(g, nbins=N, flags=flags, nstart=n, maxeval=n))
+    I.reset()
     I.run()
     I.result()
     got = I.grid()
