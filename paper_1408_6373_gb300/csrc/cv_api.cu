@@ -23,8 +23,8 @@ namespace cv {
                                                         cudaStream_t);                      \
     extern template cudaError_t launch_sample<D, double>(const SampleArgs<double> &, int,   \
                                                          cudaStream_t);                     \
-    extern template cudaError_t sample_occupancy<D, float>(int, int *);                     \
-    extern template cudaError_t sample_occupancy<D, double>(int, int *);                    \
+    extern template cudaError_t sample_occupancy<D, float>(int, bool, int *);               \
+    extern template cudaError_t sample_occupancy<D, double>(int, bool, int *);              \
     extern template cudaError_t launch_sobol<D, unsigned int>(                              \
         unsigned long long, long long, int, const PointArgs &, unsigned long long *, int,   \
         cudaStream_t);                                                                      \
@@ -46,10 +46,10 @@ static cudaError_t dispatch_sample(int ndim, const SampleArgs<Real> &a, int grid
 }
 
 template <typename Real>
-static cudaError_t dispatch_occupancy(int ndim, int nbins, int *occ)
+static cudaError_t dispatch_occupancy(int ndim, int nbins, bool pseudo, int *occ)
 {
     switch (ndim) {
-#define CV_CASE(D) case D: return sample_occupancy<D, Real>(nbins, occ);
+#define CV_CASE(D) case D: return sample_occupancy<D, Real>(nbins, pseudo, occ);
         CV_FOR_EACH_NDIM(CV_CASE)
 #undef CV_CASE
     }
@@ -192,7 +192,7 @@ extern "C" int cv_create(cv_ctx **out, int device, void *stream)
         delete ctx;
         return CV_ECUDA;
     }
-    ctx->occ.assign(2 * (CV_MAX_DIM + 1) * (CV_MAX_BINS + 1), 0);
+    ctx->occ.assign(4 * (CV_MAX_DIM + 1) * (CV_MAX_BINS + 1), 0);
     bool ok = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) == cudaSuccess;
     for (int k = 0; k < kSideStreams && ok; ++k)
         ok = cudaStreamCreateWithFlags(&ctx->side[k], cudaStreamNonBlocking) == cudaSuccess &&
@@ -489,13 +489,15 @@ static void fill_params(const cv_genz *g, GenzParams<Real> *p)
     fill_genz_params<Real>(g, p);
 }
 
-static int occupancy(cv_ctx *ctx, int ndim, int nbins, bool fp64, int *occ)
+// Resident blocks per SM of the pass that the flags choose.
+static int occupancy(cv_ctx *ctx, int ndim, int nbins, int flags, int *occ)
 {
-    int &slot = ctx->occ[((fp64 ? 1 : 0) * (CV_MAX_DIM + 1) + ndim) * (CV_MAX_BINS + 1) + nbins];
+    const bool fp64 = (flags & CV_FP64) != 0, pseudo = (flags & CV_PSEUDO) != 0;
+    int &slot = ctx->occ[(((pseudo ? 2 : 0) + (fp64 ? 1 : 0)) * (CV_MAX_DIM + 1) + ndim) * (CV_MAX_BINS + 1) + nbins];
     if (slot == 0) {
         int o = 0;
-        cudaError_t e = fp64 ? dispatch_occupancy<double>(ndim, nbins, &o)
-                             : dispatch_occupancy<float>(ndim, nbins, &o);
+        cudaError_t e = fp64 ? dispatch_occupancy<double>(ndim, nbins, pseudo, &o)
+                             : dispatch_occupancy<float>(ndim, nbins, pseudo, &o);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy query");
         slot = o > 0 ? o : 1;
     }
@@ -578,7 +580,7 @@ static int pass_grid(cv_ctx *ctx, const cv_genz *g, int nbins, int flags, long l
             }
         }
     }
-    int occ = 0, rc = occupancy(ctx, g->ndim, nbins, sizeof(Real) == 8, &occ);
+    int occ = 0, rc = occupancy(ctx, g->ndim, nbins, flags, &occ);
     if (rc) return rc;
     *grid = sample_grid(ctx, occ, n_grid, sizeof(Real) == 8);
     return CV_OK;
@@ -633,7 +635,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
                      err.c_str());
         }
     }
-    int occ = 0, rc = occupancy(ctx, g->ndim, nbins, sizeof(Real) == 8, &occ);
+    int occ = 0, rc = occupancy(ctx, g->ndim, nbins, flags, &occ);
     if (rc) return rc;
     const int grid = sample_grid(ctx, occ, n_grid, sizeof(Real) == 8);
     use_parts(grid);
@@ -963,7 +965,7 @@ static int capture_graph(cv_integral *I)
     // the occupancy query sets kernel attributes, and a run-time
     // specialisation compiles and loads a module: both before capturing
     int occ = 0;
-    int rc = occupancy(ctx, I->spec.g.ndim, I->spec.nbins, (I->spec.flags & CV_FP64) != 0, &occ);
+    int rc = occupancy(ctx, I->spec.g.ndim, I->spec.nbins, I->spec.flags, &occ);
     if (rc) return rc;
     if ((I->spec.flags & CV_JIT) && !(I->spec.flags & CV_FP64)) {
         SampleArgs<float> a;
@@ -2941,7 +2943,7 @@ static int vegas_cb_run(cv_ctx *ctx, int ndim, int ncomp, cv_integrand_dev cb, v
     a.S2 = st->S2;
     a.H = H;
     int occ = 0;
-    rc = occupancy(ctx, ndim, N, sizeof(Real) == 8, &occ);
+    rc = occupancy(ctx, ndim, N, sizeof(Real) == 8 ? CV_FP64 : 0, &occ);
     if (rc) return rc;
     pin[0] = 1;
     int aborted = 0;

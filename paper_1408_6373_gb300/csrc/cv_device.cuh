@@ -2397,10 +2397,9 @@ cudaError_t launch_sample(const SampleArgs<Real> &a, int grid, cudaStream_t s)
 }
 
 template <int NDIM, typename Real>
-cudaError_t sample_occupancy(int nbins, int *blocks_per_sm)
+cudaError_t sample_occupancy(int nbins, bool pseudo, int *blocks_per_sm)
 {
     const MapParams m = make_map(nbins, NDIM, sizeof(Real) == 8);
-    const size_t smem = sample_smem_bytes(NDIM, nbins, sizeof(Real) == 8, m.priv != 0);
     int optin = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -2415,7 +2414,11 @@ cudaError_t sample_occupancy(int nbins, int *blocks_per_sm)
         e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
         if (e != cudaSuccess) return e;
     }
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, kBlock, smem);
+    // (pseudo-random points share one histogram copy: 8 dimensions x 256 bins
+    // hold three blocks, where the Sobol pass's copies leave room for two, and
+    // take 295 us a pass of 1e7 points on them, 319 on two)
+    const size_t smem = sample_smem_bytes(NDIM, nbins, sizeof(Real) == 8, !pseudo && m.priv != 0);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, all[pseudo ? 1 : 0], kBlock, smem);
 }
 
 template <int NDIM, bool POW2>
@@ -2540,8 +2543,8 @@ cudaError_t launch_sobol(unsigned long long start, long long n, int bits, const 
                                                      cudaStream_t);                         \
     template cudaError_t cv::launch_sample<D, double>(const cv::SampleArgs<double> &, int,  \
                                                       cudaStream_t);                        \
-    template cudaError_t cv::sample_occupancy<D, float>(int, int *);                        \
-    template cudaError_t cv::sample_occupancy<D, double>(int, int *);                       \
+    template cudaError_t cv::sample_occupancy<D, float>(int, bool, int *);                  \
+    template cudaError_t cv::sample_occupancy<D, double>(int, bool, int *);                 \
     template cudaError_t cv::launch_batch_sample<D, true>(const cv::BatchSampleArgs &, int,  \
                                                           cudaStream_t);                    \
     template cudaError_t cv::launch_batch_sample<D, false>(const cv::BatchSampleArgs &, int, \

@@ -389,7 +389,7 @@ inline size_t batch_smem_bytes(int ndim, int stride) {
 template <int NDIM, typename Real>
 cudaError_t launch_sample(const SampleArgs<Real> &a, int grid, cudaStream_t s);
 template <int NDIM, typename Real>
-cudaError_t sample_occupancy(int nbins, int *blocks_per_sm);
+cudaError_t sample_occupancy(int nbins, bool pseudo, int *blocks_per_sm);
 template <int NDIM, bool POW2>
 cudaError_t launch_batch_sample(const BatchSampleArgs &b, int grid, cudaStream_t s);
 template <int NDIM>

@@ -86,10 +86,10 @@ struct DeviceGuard {
     X(31) X(32)
 
 template <typename Real>
-cudaError_t occupancy_of(int ndim, int nbins, int *occ)
+cudaError_t occupancy_of(int ndim, int nbins, bool pseudo, int *occ)
 {
     switch (ndim) {
-#define CV_NA_CASE(D) case D: return cv::sample_occupancy<D, Real>(nbins, occ);
+#define CV_NA_CASE(D) case D: return cv::sample_occupancy<D, Real>(nbins, pseudo, occ);
         CV_NA_FOR_EACH_NDIM(CV_NA_CASE)
 #undef CV_NA_CASE
     }
@@ -125,7 +125,7 @@ cudaError_t run(const cv_genz *g, int nbins, int flags, unsigned long long seed,
     a.H = H;
     a.st = st;
     int occ = 0;
-    cudaError_t e = occupancy_of<Real>(g->ndim, nbins, &occ);
+    cudaError_t e = occupancy_of<Real>(g->ndim, nbins, a.gen == cv::kGenPseudo, &occ);
     if (e != cudaSuccess) return e;
     const long long nblk = (nmax + 63) / 32;
     long long grid = (nblk + (long long)cv::kWarpsPerBlock * 16 - 1) / ((long long)cv::kWarpsPerBlock * 16);
