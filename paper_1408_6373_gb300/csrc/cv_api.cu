@@ -9,6 +9,7 @@
 #include <set>
 #include <vector>
 
+#include "cv_grid.h"
 #include "cv_internal.cuh"
 
 #define CV_FOR_EACH_NDIM(X)                                                                  \
@@ -505,26 +506,16 @@ static int occupancy(cv_ctx *ctx, int ndim, int nbins, int flags, int *occ)
     return CV_OK;
 }
 
-// Blocks for a pass over n points: as many CTAs per SM as leave every warp
-// about ten 32-point blocks, at most one full wave of resident CTAs; a pass
-// too small for one CTA on every SM spreads over the SMs, six blocks per
-// CTA.  A CTA costs its prologue (the grid table, the histogram copies) and
-// a partial row that the refinement adds, so more CTAs than the points need
-// are not free; us per iteration (6 dimensions, 2 components, 64 bins), on
-// 76 / 152 / 304 / 456 CTAs: 16.0 / 15.5 / 16.4 / 17.4 for 3e4 points,
-// 23.0 / 19.2 / 19.1 / 21.0 for 3e5, 44 / 29.0 / 24.8 / 26.2 for 1e6,
-// 104 / 59 / 41.7 / 39.0 for 3e6.  An FP64 pass takes a block for each of
-// four warps of a CTA: its time is the SM's FP64 lanes, which all its warps
-// share (and the refinement's is the rows it adds, so not one warp per CTA):
-// 3 dimensions, 50 bins, 1e4 points 17.2 us an iteration, 18.8 with one or
-// two and 18.5 with eight.
-static int sample_grid(cv_ctx *ctx, int occ, long long n, bool fp64)
+// Blocks for a pass over n points with the parameters, map and generator of a.
+template <typename Real>
+static int sample_grid(cv_ctx *ctx, int occ, long long n, const SampleArgs<Real> &a)
 {
-    const long long nblk = (n + 63) / 32, sms = ctx->sms;
-    const long long small = fp64 ? (nblk + 3) / 4 : (nblk + 5) / 6;
-    if (small < sms) return small < 1 ? 1 : (int)small;
-    const long long per_sm = nblk / (sms * kWarpsPerBlock * 10);
-    return (int)(sms * std::min<long long>(std::max<long long>(per_sm, 1), occ));
+    PassKind k;
+    k.fp64 = sizeof(Real) == 8;
+    k.pseudo = a.gen == kGenPseudo;
+    k.block_hist = !k.fp64 && !k.pseudo && !a.map.pow2;
+    k.chain = (long long)a.g.delay * a.g.ncomp;
+    return sampling_blocks(ctx->sms, occ, n, k);
 }
 
 // Blocks for a materialised pass over n points (bound by HBM, so a full wave
@@ -564,25 +555,25 @@ static void parts_args(const PassParts *pp, int grid, double **S, void **H, unsi
 template <typename Real>
 static int pass_grid(cv_ctx *ctx, const cv_genz *g, int nbins, int flags, long long n_grid, int *grid)
 {
+    SampleArgs<Real> a;
+    memset(&a, 0, sizeof(a));
+    fill_params<Real>(g, &a.g);
+    a.nbins = nbins;
+    a.map = make_map(nbins, g->ndim, sizeof(Real) == 8);
+    set_generator(&a, g->ndim, flags, 0);
     if constexpr (sizeof(Real) == 4) {
         if (flags & CV_JIT) {
-            SampleArgs<float> a;
-            memset(&a, 0, sizeof(a));
-            fill_params<float>(g, &a.g);
-            a.nbins = nbins;
-            a.map = make_map(nbins, g->ndim, false);
-            set_generator(&a, g->ndim, flags, 0);
             JitKernel k;
             std::string err;
             if (jit_sample_kernel(ctx->device, a, g->ndim, a.map.pow2 != 0, min_blocks_f32(g->ndim), &k, &err) == 0) {
-                *grid = sample_grid(ctx, k.occ, n_grid, false);
+                *grid = sample_grid(ctx, k.occ, n_grid, a);
                 return CV_OK;
             }
         }
     }
     int occ = 0, rc = occupancy(ctx, g->ndim, nbins, flags, &occ);
     if (rc) return rc;
-    *grid = sample_grid(ctx, occ, n_grid, sizeof(Real) == 8);
+    *grid = sample_grid(ctx, occ, n_grid, a);
     return CV_OK;
 }
 
@@ -623,7 +614,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
             JitKernel k;
             std::string err;
             if (jit_sample_kernel(ctx->device, a, g->ndim, a.map.pow2 != 0, min_blocks_f32(g->ndim), &k, &err) == 0) {
-                const int grid = sample_grid(ctx, k.occ, n_grid, false);
+                const int grid = sample_grid(ctx, k.occ, n_grid, a);
                 use_parts(grid);
                 const int tk = timer_begin(ctx);
                 cudaError_t e = launch_jit_sample(k, a, grid, ctx->stream);
@@ -637,7 +628,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
     }
     int occ = 0, rc = occupancy(ctx, g->ndim, nbins, flags, &occ);
     if (rc) return rc;
-    const int grid = sample_grid(ctx, occ, n_grid, sizeof(Real) == 8);
+    const int grid = sample_grid(ctx, occ, n_grid, a);
     use_parts(grid);
     const int tk = timer_begin(ctx);
     cudaError_t e = dispatch_sample<Real>(g->ndim, a, grid, ctx->stream);
