@@ -501,8 +501,9 @@ void cv_integral_destroy(cv_integral *I);
  * the per-warp histograms in shared memory (10 * ndim * nbins * 4 bytes
  * <= 227 KiB, e.g. 32 x 128 or 20 x 256).  An integral's points are cut
  * into tiles by a rule that depends on that integral alone (at most 32
- * tiles per iteration, 2^11 .. cap points each; CUBAGPU_TILE, points,
- * forces one size), and each tile leaves its sums and histogram as
+ * tiles per iteration, 2^11 .. cap points each, the cap's size up to 512
+ * tiles, then up to 2^16 points; CUBAGPU_TILE, points, forces one size), and
+ * each tile leaves its sums and histogram as
  * partial rows that the refinement and combination add in tile order (no
  * floating-point atomics), so an integral's result is the same alone, in
  * any batch and on every run, bit for bit, for the same tile cap and split.

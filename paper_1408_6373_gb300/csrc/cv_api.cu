@@ -1593,21 +1593,6 @@ static cudaError_t dispatch_batch_occupancy(int ndim, bool pow2, int stride, int
 }
 }  // namespace cv
 
-// Tile size, in 32-point blocks, of one integral's iteration of n points:
-// the smallest power of two >= 64 blocks that cuts the iteration into at
-// most `split` tiles, capped at `cap` blocks.  It depends on the integral
-// alone, so a batch or a serving round never changes how an integral's
-// points are grouped and summed.  A tile is shared evenly by a CTA's eight
-// warps, so the points each thread takes from a tile are tile / 8: split
-// and cap set the points per thread (the autotuner picks both).
-static int tile_blocks_for(long long n, int cap, int split)
-{
-    const long long blocks = (n + 31) / 32 + 1;
-    long long t = 64;
-    while (t < cap && t * split < blocks) t <<= 1;
-    return (int)t;
-}
-
 // Defaults of the rule.  A tile costs ~5 us of a CTA besides its points,
 // and a launch's end is as long as its last tiles, so the best size is
 // between: every tile 2^11 / 2^12 / 2^13 / 2^14 / 2^15 points took 9.1 / 7.2
@@ -1729,6 +1714,7 @@ static int grow_device(cv_ctx *ctx, T **p, size_t *cap, size_t need, const char 
 
 // Histogram row stride of a tile partial: ndim nbins floats rounded up to
 // a multiple of 4 (16-byte aligned rows).
+constexpr size_t kPartFloats = 4ull * 0xffffffffull;  // (offsets are counted in fours)
 static unsigned tile_row_floats(int ndim, int nbins) { return ((unsigned)(ndim * nbins) + 3u) & ~3u; }
 
 // Generate every tile of every iteration for the current tile sizes.
@@ -1752,7 +1738,7 @@ static int batch_build_tiles(cv_batch *B, int only_first_iteration)
                 if (B->item_class[i] != (int)c || j >= B->jmax[i]) continue;
                 TileParts &tp = tparts[(size_t)j * B->count + i];
                 tp.row0 = (int)(tiles.size() - it0);
-                tp.hoff0 = (unsigned)hf;
+                tp.hoff0 = (unsigned)(hf / 4);
                 tp.stride = (int)tile_row_floats(B->specs[i].g.ndim, B->specs[i].nbins);
                 const cv_spec &sp = B->specs[i];
                 // start index and size of iteration j (the device follows the same plan)
@@ -1769,7 +1755,7 @@ static int batch_build_tiles(cv_batch *B, int only_first_iteration)
                     t.q0 = q;
                     t.st = B->states[i];
                     t.row = (int)(tiles.size() - it0);
-                    t.hoff = (unsigned)hf;
+                    t.hoff = (unsigned)(hf / 4);
                     hf += (size_t)tp.stride;
                     tiles.push_back(t);
                     ++tp.count;
@@ -1782,7 +1768,7 @@ static int batch_build_tiles(cv_batch *B, int only_first_iteration)
         rows_max = std::max(rows_max, tiles.size() - it0);
         floats_max = std::max(floats_max, hf);
     }
-    if (floats_max > 0xffffffffull) return fail_msg(ctx, CV_ENOMEM, "tile partials beyond 2^32 floats per iteration");
+    if (floats_max > kPartFloats) return fail_msg(ctx, CV_ENOMEM, "tile partials beyond 2^34 floats per iteration");
     {
         int rc = grow_device(ctx, &B->d_part_S, &B->part_rows_cap, rows_max * 2 * CV_MAX_COMP, "tile sum partials");
         if (!rc) rc = grow_device(ctx, &B->d_part_H, &B->part_floats_cap, floats_max, "tile histogram partials");
@@ -2436,9 +2422,9 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
         Tile &t = all[k];
         TileParts &tp = S->h_tparts[t.item];
         const unsigned stride = S->slot_stride[t.item];
-        if (k == 0 || all[k - 1].item != t.item) tp = TileParts{(int)k, 0, (unsigned)hf, (int)stride};
+        if (k == 0 || all[k - 1].item != t.item) tp = TileParts{(int)k, 0, (unsigned)(hf / 4), (int)stride};
         t.row = (int)k;
-        t.hoff = (unsigned)hf;
+        t.hoff = (unsigned)(hf / 4);
         hf += stride;
         ++tp.count;
     }
@@ -2449,7 +2435,7 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
             t += c.tiles.size();
         }
     }
-    if (hf > 0xffffffffull) return fail_msg(ctx, CV_ENOMEM, "tile partials beyond 2^32 floats per round");
+    if (hf > kPartFloats) return fail_msg(ctx, CV_ENOMEM, "tile partials beyond 2^34 floats per round");
     {
         int rc = grow_device(ctx, &S->d_part_S, &S->part_rows_cap, all.size() * 2 * CV_MAX_COMP, "tile sum partials");
         if (!rc) rc = grow_device(ctx, &S->d_part_H, &S->part_floats_cap, hf, "tile histogram partials");

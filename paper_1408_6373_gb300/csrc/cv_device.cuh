@@ -1669,7 +1669,7 @@ k_batch_sample(const BatchSampleArgs B)
             }
             // (warp copies summed in warp order, then cleared)
             const int N = A.nbins;
-            float *ph = B.part_S ? B.part_H + tile.hoff : nullptr;
+            float *ph = B.part_S ? B.part_H + 4 * (size_t)tile.hoff : nullptr;
             if (POW2 && ph && N == stride) {
                 // (N a multiple of 32: rows and copies are 16-byte aligned)
                 float4 *ph4 = reinterpret_cast<float4 *>(ph);

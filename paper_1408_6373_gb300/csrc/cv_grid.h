@@ -1,5 +1,5 @@
-// cv_grid.h -- the number of blocks of a sampling pass.  Plain C++, so that
-// the rule can be evaluated without a GPU.
+// cv_grid.h -- the number of blocks of a sampling pass, and the tiles of a
+// batched one.  Plain C++, so that the rules can be evaluated without a GPU.
 #pragma once
 
 namespace cv {
@@ -60,6 +60,26 @@ inline int sampling_blocks(int sms, int occ, long long n, const PassKind &k)
     if (per_sm < 1) per_sm = 1;
     if (per_sm > occ) per_sm = occ;
     return (int)(per_sm * sms);
+}
+
+// Tile size, in 32-point blocks, of one integral's iteration of n points:
+// the smallest power of two >= 64 blocks that cuts the iteration into at
+// most `split` tiles, capped at `cap` blocks.  It depends on the integral
+// alone, so a batch or a serving round never changes how an integral's
+// points are grouped and summed.  A tile is shared evenly by a CTA's eight
+// warps, so the points each thread takes from a tile are tile / 8: split
+// and cap set the points per thread (the autotuner picks both).  Every tile
+// leaves a histogram row of its own, so an iteration of more than 512 tiles
+// at the cap takes larger ones, up to 2^16 points: from there on the rows are
+// what bounds how many large integrals fit the device, and a CTA has so many
+// tiles that their size no longer shows.
+inline int tile_blocks_for(long long n, int cap, int split)
+{
+    const long long blocks = (n + 31) / 32 + 1;
+    long long t = 64;
+    while (t < cap && t * split < blocks) t <<= 1;
+    while (t < 2048 && t * 512 < blocks) t <<= 1;
+    return (int)t;
 }
 
 }  // namespace cv

@@ -348,12 +348,12 @@ struct alignas(16) Tile {
     unsigned long long q0;
     const DevState *st;
     int row;                        // row of BatchSampleArgs::part_S
-    unsigned hoff;                  // first float of its [ndim][nbins] rows in part_H
+    unsigned hoff;                  // its [ndim][nbins] rows start at float 4 hoff of part_H
 };
 
 // The partial rows of one integral's tiles in one iteration: count
 // consecutive sum rows from row0, and histogram rows of `stride` floats
-// (ndim nbins rounded up to a multiple of 4) from float hoff0.
+// (ndim nbins rounded up to a multiple of 4) from float 4 hoff0.
 struct TileParts {
     int row0;
     int count;
@@ -369,7 +369,7 @@ struct BatchSampleArgs {
     int *counter;                   // next tile to take (zero before the launch)
     // Deterministic reduction (part_S non-null): tile t writes its sums to
     // part_S[t.row][2 c + {0, 1}] and its histogram, by slot, to part_H +
-    // t.hoff, no atomics; the batched refinement and combination add an
+    // 4 t.hoff, no atomics; the batched refinement and combination add an
     // integral's rows in tile order.  Null: FP64 atomics into the
     // integral's state and histogram.
     double *part_S;

@@ -906,7 +906,7 @@ __global__ void __launch_bounds__(256) k_batch_refine(const BatchItem *items, co
         // the histogram of the integral's tiles, rows added in tile order
         const TileParts tp = parts[ax.x];
         CombineArgs pa;
-        pa.part_H = part_H + tp.hoff0;
+        pa.part_H = part_H + 4 * (size_t)tp.hoff0;
         pa.part_G = tp.count;
         pa.part_nh = tp.stride;
         pa.part_f32 = 1;

@@ -50,3 +50,24 @@ def test_iterations_match_oracle(ctx, ndim, bins):
             check_fp32_iteration(I[j], V[j], ob, n, what=(ndim, N, n, j))
     B1.close()
     B2.close()
+
+
+def test_rows_beyond_2_to_32_floats(ctx):
+    # 1800 integrals of 489 tiles, rows of 5120 floats: 4.5e9 floats of partial
+    # rows, and the last integral's (behind them) the same bits as alone
+    ndim, N, n = 32, 160, 16000000
+    if torch.cuda.mem_get_info()[0] < 40 << 30:
+        pytest.skip("needs 40 GB")
+    g = cg.genz(ndim, [O.C0], 0.1 * np.ones((1, ndim)), 0.5 * np.ones((1, ndim)))
+    last = cg.spec(cg.genz(ndim, [O.GAUSSIAN], 0.3 * np.ones((1, ndim)), 0.4 * np.ones((1, ndim))), nbins=N,
+                   nstart=n, maxeval=n)
+    B = ctx.batch([cg.spec(g, nbins=N, nstart=n, maxeval=n)] * 1799 + [last])
+    B.run()
+    r, grid = B.results()[-1], B.grid(1799)
+    B.close()
+    A = ctx.batch([last])
+    A.run()
+    a = A.results()[0]
+    assert r.integral[0] == a.integral[0] and r.error[0] == a.error[0]
+    assert np.array_equal(A.grid(0), grid)
+    A.close()

@@ -1,4 +1,4 @@
-"""The number of blocks of a sampling pass (cv_grid.h, compiled for the host).
+"""The rules of cv_grid.h, compiled for the host: blocks of a pass, tiles of a batch.
 
 For every kind of pass and 152 SMs: at least one block, at most one wave, never
 fewer for more points; and where a point costs a warp's time rather than the
@@ -61,6 +61,38 @@ def test_sampling_blocks(tmp_path):
         pytest.skip("no g++")
     src, exe = tmp_path / "grid.cpp", tmp_path / "grid"
     src.write_text(PROGRAM)
+    subprocess.run(["g++", "-std=c++17", "-O2", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    res = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert res.returncode == 0, res.stdout
+
+
+TILES = r"""
+#include <initializer_list>
+#include <cstdio>
+#include "cv_grid.h"
+int main()
+{
+    int bad = 0;
+    for (int cap : {256, 1024, 2048, 4096})
+        for (int split : {8, 16, 32})
+            for (long long n = 1; n < (1ll << 45); n += 1 + n / 16) {
+                const long long blocks = (n + 31) / 32 + 1, t = cv::tile_blocks_for(n, cap, split);
+                const long long tiles = (blocks + t - 1) / t, most = (blocks + 2047) / 2048;
+                const bool ok = t >= 64 && !(t & (t - 1)) && t <= (cap > 2048 ? cap : 2048) &&
+                                tiles <= (most > 512 ? most : 512) && (blocks > 512 * (long long)cap || t <= cap);
+                if (!ok && bad++ < 10) printf("n %lld cap %d split %d: tiles of %lld blocks\n", n, cap, split, t);
+            }
+    return bad ? 1 : 0;
+}
+"""
+
+
+def test_tiles_leave_few_rows(tmp_path):
+    # at most 512 rows an iteration, or those of tiles of 2^16 points
+    if shutil.which("g++") is None:
+        pytest.skip("no g++")
+    src, exe = tmp_path / "tiles.cpp", tmp_path / "tiles"
+    src.write_text(TILES)
     subprocess.run(["g++", "-std=c++17", "-O2", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     res = subprocess.run([str(exe)], capture_output=True, text=True)
     assert res.returncode == 0, res.stdout
