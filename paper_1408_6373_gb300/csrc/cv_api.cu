@@ -1604,12 +1604,54 @@ static cudaError_t dispatch_batch_occupancy(int ndim, bool pow2, int stride, int
 // points for the same SMs, so its tiles stop at 2^13 (21.0 ms; before: 36.9).
 constexpr int kTileSplit = 32, kBatchTileCap = 1024, kServeTileCap = 256;
 
-// The order in which a launch hands its tiles out: the largest first (the
-// short ones then fill the queue's end), an integral's equal tiles
-// together, so that a CTA that takes several stages the integral once.
-static void order_tiles(Tile *first, Tile *last)
+// Consecutive tiles of one size of one integral; their partial rows follow
+// one another, `step` fours of floats apart.
+struct TileRun {
+    Tile first;
+    int count;
+    unsigned step;
+};
+
+// The tiles of blocks [qa, qb) in sizes of TB, with rows from `row` and
+// histogram float `hf` on; returns their number.
+static int add_tiles(std::vector<TileRun> *runs, int item, const DevState *st, unsigned long long qa,
+                     unsigned long long qb, int TB, size_t row, size_t hf, unsigned stride)
 {
-    std::stable_sort(first, last, [](const Tile &x, const Tile &y) { return x.nblk > y.nblk; });
+    const int full = (int)((qb - qa) / (unsigned long long)TB), rest = (int)((qb - qa) % (unsigned long long)TB);
+    Tile t;
+    t.item = item;
+    t.nblk = TB;
+    t.q0 = qa;
+    t.st = st;
+    t.row = (int)row;
+    t.hoff = (unsigned)(hf / 4);
+    if (full) runs->push_back({t, full, stride / 4});
+    t.nblk = rest;
+    t.q0 += (unsigned long long)full * (unsigned long long)TB;
+    t.row += full;
+    t.hoff = (unsigned)((hf + (size_t)full * stride) / 4);
+    if (rest) runs->push_back({t, 1, stride / 4});
+    return full + (rest ? 1 : 0);
+}
+
+// Append the runs' tiles in the order in which a launch hands them out: the
+// largest first (the short ones then fill the queue's end), an integral's
+// equal tiles together, so that a CTA that takes several stages the integral
+// once.  (The runs are sorted, two for an integral, not the tiles: 512
+// integrals' 82 thousand tiles took 0.5 ms of the batch's creation.)
+static void emit_tiles(std::vector<TileRun> *runs, std::vector<Tile> *out)
+{
+    std::stable_sort(runs->begin(), runs->end(),
+                     [](const TileRun &x, const TileRun &y) { return x.first.nblk > y.first.nblk; });
+    for (const TileRun &r : *runs) {
+        Tile t = r.first;
+        for (int i = 0; i < r.count; ++i) {
+            out->push_back(t);
+            t.q0 += (unsigned long long)t.nblk;
+            ++t.row;
+            t.hoff += r.step;
+        }
+    }
 }
 
 // The device memory of one integral of a batch or a server: state, FP64
@@ -1722,6 +1764,7 @@ static int batch_build_tiles(cv_batch *B, int only_first_iteration)
 {
     cv_ctx *ctx = B->ctx;
     std::vector<Tile> tiles;
+    std::vector<TileRun> runs;
     B->plan.clear();
     const int J = only_first_iteration ? 1 : B->J;
     int counter = 0;
@@ -1731,13 +1774,14 @@ static int batch_build_tiles(cv_batch *B, int only_first_iteration)
     size_t rows_max = 0, floats_max = 0;
     for (int j = 0; j < J; ++j) {
         const size_t it0 = tiles.size();
-        size_t hf = 0;
+        size_t rows = 0, hf = 0;
         for (size_t c = 0; c < B->classes.size(); ++c) {
             const int off = (int)tiles.size();
+            runs.clear();
             for (int i = 0; i < B->count; ++i) {
                 if (B->item_class[i] != (int)c || j >= B->jmax[i]) continue;
                 TileParts &tp = tparts[(size_t)j * B->count + i];
-                tp.row0 = (int)(tiles.size() - it0);
+                tp.row0 = (int)rows;
                 tp.hoff0 = (unsigned)(hf / 4);
                 tp.stride = (int)tile_row_floats(B->specs[i].g.ndim, B->specs[i].nbins);
                 const cv_spec &sp = B->specs[i];
@@ -1748,21 +1792,12 @@ static int batch_build_tiles(cv_batch *B, int only_first_iteration)
                 const int TB = B->tile_fixed ? B->tile_fixed : tile_blocks_for((long long)n, B->tile_cap, B->tile_split);
                 // (tiles start on even 32-point blocks: see run_steps)
                 const unsigned long long qa = (s >> 5) & ~1ull, qb = (s + n + 31) >> 5;
-                for (unsigned long long q = qa; q < qb; q += (unsigned long long)TB) {
-                    Tile t;
-                    t.item = i;
-                    t.nblk = (int)(qb - q < (unsigned long long)TB ? qb - q : (unsigned long long)TB);
-                    t.q0 = q;
-                    t.st = B->states[i];
-                    t.row = (int)(tiles.size() - it0);
-                    t.hoff = (unsigned)(hf / 4);
-                    hf += (size_t)tp.stride;
-                    tiles.push_back(t);
-                    ++tp.count;
-                }
+                tp.count = add_tiles(&runs, i, B->states[i], qa, qb, TB, rows, hf, (unsigned)tp.stride);
+                rows += (size_t)tp.count;
+                hf += (size_t)tp.count * (size_t)tp.stride;
             }
+            emit_tiles(&runs, &tiles);
             const int nt = (int)tiles.size() - off;
-            order_tiles(tiles.data() + off, tiles.data() + tiles.size());
             if (nt > 0) B->plan.push_back({j, (int)c, off, nt, counter++});
         }
         rows_max = std::max(rows_max, tiles.size() - it0);
@@ -2373,7 +2408,7 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
     }
     const int nlive = (int)live.size();
     // tiles grouped by dimension class
-    struct Cls { int ndim; bool pow2; int stride; std::vector<Tile> tiles; };
+    struct Cls { int ndim; bool pow2; int stride; std::vector<TileRun> runs; size_t ntiles; };
     std::vector<Cls> cls;
     int64_t round_samples = 0;
     for (const Request &r : live) {
@@ -2384,7 +2419,7 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
         for (Cls &k : cls)
             if (k.ndim == ndim && k.pow2 == p2) c = &k;
         if (!c) {
-            cls.push_back({ndim, p2, r.spec.nbins, {}});
+            cls.push_back({ndim, p2, r.spec.nbins, {}, 0});
             c = &cls.back();
         }
         c->stride = std::max(c->stride, r.spec.nbins);
@@ -2393,18 +2428,13 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
         const long long tb = S->opts.tile_points > 0 ? std::max(1, S->opts.tile_points / 32)
                                                      : tile_blocks_for((long long)n, kServeTileCap, kTileSplit);
         const unsigned long long qa = (s >> 5) & ~1ull, qb = (s + n + 31) >> 5;
-        for (unsigned long long q = qa; q < qb; q += (unsigned long long)tb) {
-            Tile t;
-            t.item = r.slot;
-            t.nblk = (int)std::min<unsigned long long>(qb - q, (unsigned long long)tb);
-            t.q0 = q;
-            t.st = (const DevState *)((const char *)S->arena_mem + r.off);
-            c->tiles.push_back(t);
-        }
+        // (rows from 0: placed below, class after class)
+        c->ntiles += (size_t)add_tiles(&c->runs, r.slot, (const DevState *)((const char *)S->arena_mem + r.off), qa, qb,
+                                       (int)tb, 0, 0, S->slot_stride[r.slot]);
         round_samples += (int64_t)n;
     }
     size_t ntiles = 0;
-    for (const Cls &c : cls) ntiles += c.tiles.size();
+    for (const Cls &c : cls) ntiles += c.ntiles;
     if (ntiles > S->tiles_cap) {
         if (S->d_tiles) cudaFree(S->d_tiles);
         S->d_tiles = nullptr;
@@ -2414,26 +2444,23 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
     }
     std::vector<Tile> all;
     all.reserve(ntiles);
-    for (const Cls &c : cls) all.insert(all.end(), c.tiles.begin(), c.tiles.end());
-    // the round's partial rows: tile k of the queue at row k, its histogram
-    // after the previous tiles'; a request's tiles are consecutive
-    size_t hf = 0;
-    for (size_t k = 0; k < all.size(); ++k) {
-        Tile &t = all[k];
-        TileParts &tp = S->h_tparts[t.item];
-        const unsigned stride = S->slot_stride[t.item];
-        if (k == 0 || all[k - 1].item != t.item) tp = TileParts{(int)k, 0, (unsigned)(hf / 4), (int)stride};
-        t.row = (int)k;
-        t.hoff = (unsigned)(hf / 4);
-        hf += stride;
-        ++tp.count;
-    }
-    {
-        Tile *t = all.data();
-        for (const Cls &c : cls) {
-            order_tiles(t, t + c.tiles.size());
-            t += c.tiles.size();
+    // the round's partial rows: the requests' tiles one after another, class
+    // after class, each histogram row after the previous tile's
+    size_t row = 0, hf = 0;
+    for (Cls &c : cls) {
+        int last = -1;
+        for (TileRun &t : c.runs) {
+            TileParts &tp = S->h_tparts[t.first.item];
+            const unsigned stride = S->slot_stride[t.first.item];
+            if (t.first.item != last) tp = TileParts{(int)row, 0, (unsigned)(hf / 4), (int)stride};
+            last = t.first.item;
+            t.first.row = (int)row;
+            t.first.hoff = (unsigned)(hf / 4);
+            row += (size_t)t.count;
+            hf += (size_t)t.count * stride;
+            tp.count += t.count;
         }
+        emit_tiles(&c.runs, &all);
     }
     if (hf > kPartFloats) return fail_msg(ctx, CV_ENOMEM, "tile partials beyond 2^34 floats per round");
     {
@@ -2456,10 +2483,10 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
         size_t o = 0;
         for (size_t i = 0; i < cls.size(); ++i) {
             offs[i] = o;
-            o += cls[i].tiles.size();
+            o += cls[i].ntiles;
         }
     }
-    std::sort(order.begin(), order.end(), [&](int x, int y) { return cls[x].tiles.size() > cls[y].tiles.size(); });
+    std::sort(order.begin(), order.end(), [&](int x, int y) { return cls[x].ntiles > cls[y].ntiles; });
     CV_CUDA(ctx, cudaEventRecord(S->ev_fork, S->stream));
     for (int k = 0; k < kSideStreams; ++k) CV_CUDA(ctx, cudaStreamWaitEvent(S->side[k], S->ev_fork, 0));
     int used = 0;
@@ -2475,7 +2502,7 @@ int server_round(cv_server *S, std::vector<Request> &live, Arena &arena,
         BatchSampleArgs a;
         a.items = S->d_items;
         a.tiles = S->d_tiles + off;
-        a.ntiles = (int)c.tiles.size();
+        a.ntiles = (int)c.ntiles;
         a.stride = c.stride;
         a.counter = S->d_counters + (c.pow2 ? 1 : 0) * (CV_MAX_DIM + 1) + c.ndim;
         a.part_S = S->d_part_S;
