@@ -457,10 +457,13 @@ __device__ __forceinline__ double genz_f64(const GenzParams<double> &g, const do
         for (int d = 0; d < NDIM; ++d) s = __fma_rn(I::template p0<C>(g, d), x[d], s);
         s += 1.0;
         const double r = __drcp_rn(s);
-        const double w = r > 0.0 ? __fma_rn(-s, r, 1.0) : 0.0;  // (s may be infinite)
+        // (no residual where s or r is infinite, and no low part to add where
+        // the power is: by the bits, an FP64 comparison being the dearer way)
+        const unsigned hr = (unsigned)__double2hiint(r) & 0x7fffffffu;
+        const double w = hr - 1u < 0x7fefffffu ? __fma_rn(-s, r, 1.0) : 0.0;
         double fl;
         const double fh = ipow_df<NDIM + 1>(r, r * w, fl);
-        return fh + fl;
+        return (~__double2hiint(fl) & 0x7ff00000) ? fh + fl : fh;
     }
     case CV_GAUSSIAN:
 #pragma unroll
