@@ -506,15 +506,14 @@ static int occupancy(cv_ctx *ctx, int ndim, int nbins, int flags, int *occ)
     return CV_OK;
 }
 
-// Blocks for a pass over n points with the parameters, map and generator of a.
-template <typename Real>
-static int sample_grid(cv_ctx *ctx, int occ, long long n, const SampleArgs<Real> &a)
+// Blocks for a pass over n points of g.
+static int sample_grid(cv_ctx *ctx, int occ, long long n, const cv_genz *g, int nbins, int flags)
 {
     PassKind k;
-    k.fp64 = sizeof(Real) == 8;
-    k.pseudo = a.gen == kGenPseudo;
-    k.block_hist = !k.fp64 && !k.pseudo && !a.map.pow2;
-    k.chain = (long long)a.g.delay * a.g.ncomp;
+    k.fp64 = (flags & CV_FP64) != 0;
+    k.pseudo = (flags & CV_PSEUDO) != 0;
+    k.block_hist = !k.fp64 && !k.pseudo && !make_map(nbins, g->ndim, false).pow2;
+    k.chain = (long long)g->delay * g->ncomp;
     return sampling_blocks(ctx->sms, occ, n, k);
 }
 
@@ -555,25 +554,25 @@ static void parts_args(const PassParts *pp, int grid, double **S, void **H, unsi
 template <typename Real>
 static int pass_grid(cv_ctx *ctx, const cv_genz *g, int nbins, int flags, long long n_grid, int *grid)
 {
-    SampleArgs<Real> a;
-    memset(&a, 0, sizeof(a));
-    fill_params<Real>(g, &a.g);
-    a.nbins = nbins;
-    a.map = make_map(nbins, g->ndim, sizeof(Real) == 8);
-    set_generator(&a, g->ndim, flags, 0);
     if constexpr (sizeof(Real) == 4) {
         if (flags & CV_JIT) {
+            SampleArgs<float> a;
+            memset(&a, 0, sizeof(a));
+            fill_params<float>(g, &a.g);
+            a.nbins = nbins;
+            a.map = make_map(nbins, g->ndim, false);
+            set_generator(&a, g->ndim, flags, 0);
             JitKernel k;
             std::string err;
             if (jit_sample_kernel(ctx->device, a, g->ndim, a.map.pow2 != 0, min_blocks_f32(g->ndim), &k, &err) == 0) {
-                *grid = sample_grid(ctx, k.occ, n_grid, a);
+                *grid = sample_grid(ctx, k.occ, n_grid, g, nbins, flags);
                 return CV_OK;
             }
         }
     }
     int occ = 0, rc = occupancy(ctx, g->ndim, nbins, flags, &occ);
     if (rc) return rc;
-    *grid = sample_grid(ctx, occ, n_grid, a);
+    *grid = sample_grid(ctx, occ, n_grid, g, nbins, flags);
     return CV_OK;
 }
 
@@ -614,7 +613,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
             JitKernel k;
             std::string err;
             if (jit_sample_kernel(ctx->device, a, g->ndim, a.map.pow2 != 0, min_blocks_f32(g->ndim), &k, &err) == 0) {
-                const int grid = sample_grid(ctx, k.occ, n_grid, a);
+                const int grid = sample_grid(ctx, k.occ, n_grid, g, nbins, flags);
                 use_parts(grid);
                 const int tk = timer_begin(ctx);
                 cudaError_t e = launch_jit_sample(k, a, grid, ctx->stream);
@@ -628,7 +627,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
     }
     int occ = 0, rc = occupancy(ctx, g->ndim, nbins, flags, &occ);
     if (rc) return rc;
-    const int grid = sample_grid(ctx, occ, n_grid, a);
+    const int grid = sample_grid(ctx, occ, n_grid, g, nbins, flags);
     use_parts(grid);
     const int tk = timer_begin(ctx);
     cudaError_t e = dispatch_sample<Real>(g->ndim, a, grid, ctx->stream);
