@@ -2991,7 +2991,8 @@ static int vegas_cb_run(cv_ctx *ctx, int ndim, int ncomp, cv_integrand_dev cb, v
         SampleArgs<Real> b = a;
         b.start = s0;
         b.n = m;
-        // (the same grid as a fused pass: the kernels share its occupancy)
+        // (mat_grid over the fused kernel's occupancy; it never falls with m, so
+        // the rows for a whole tile hold every pass's)
         return dispatch_matpass<Real>(ndim, false, b, mat_grid(ctx, occ, m), s, &grid_used);
     };
     if (e == cudaSuccess && jmax > 0) e = store(start, sp.nstart < tile ? sp.nstart : tile);

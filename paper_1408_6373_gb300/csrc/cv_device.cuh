@@ -1262,7 +1262,7 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
 }
 
 // The FP32 pass for N = 2^L >= 32 when the warps' histogram copies do not fit
-// (256 bins from 7 dimensions on, 128 from 22): one copy per block, and
+// (copies_fit: 256 bins from 12 dimensions on, 128 from 23): one copy per block, and
 // every axis's row belongs to one warp, which alone updates it, without
 // atomics (a compare-and-swap loop on this GPU) and without conflicts.  The
 // block's eight warps evaluate eight consecutive 32-point blocks a round
@@ -1726,10 +1726,11 @@ k_matpass(const __grid_constant__ SampleArgs<Real> A)
     sample_pass<NDIM, Real, POW2, MatIntegrand<Real, MODE>>(A);
 }
 
-// ---- materialised samples, FP32, dimension-major, N = 2^L >= 32
-// The two passes of the common case as kernels of their own: the store
-// pass is bound by HBM writes and the accumulate pass by its reads, so both
-// keep to the instructions the point needs (no integrand, no runtime
+// ---- materialised samples, FP32, N = 2^L >= 32
+// The two passes of the common case as kernels of their own (the store pass
+// dimension-major, the accumulate pass in both layouts): the store pass is
+// bound by HBM writes, the accumulate pass by its instructions and latency,
+// so both keep to the instructions the point needs (no integrand, no runtime
 // layout or component loops).
 
 // Asynchronous 4-byte copies global -> shared (cp.async; bytes = 0 copies

@@ -179,7 +179,8 @@ struct MapParams {
     unsigned sA;                    // byte offset of the bin's grid entry = word >> sA, sA = 29 - L
     int G;                          // the fraction sits 2^-G below the mantissa's top (G = max(0, L - 6))
     int priv;                       // per-warp f^2 histograms updated without atomics, in this
-                                    // many steps (hist_phases); 0: shared-memory atomics
+                                    // many steps (hist_phases); 0: one copy per block, its axes
+                                    // owned by warps (FP32, pow2) or updated with atomics
 };
 
 #if defined(__CUDACC__)

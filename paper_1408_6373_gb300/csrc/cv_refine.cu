@@ -4,7 +4,7 @@
 // Sect. 3.2.2): per axis, smooth the f^2 histogram over neighbouring bins,
 // compress it with exponent 1.5, and move the N-1 interior edges so every
 // new bin holds an equal share of the compressed weight.  One CTA per axis;
-// the order of every FP64 operation is fixed so the result is reproducible.
+// the order of every rounded operation is fixed so the result is reproducible.
 //
 // Combination: per component, the iteration result I_j = S1/n and
 // var_j = (S2/n - I_j^2)/(n-1) are folded into the inverse-variance weighted
