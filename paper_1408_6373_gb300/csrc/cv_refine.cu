@@ -359,7 +359,7 @@ __device__ __forceinline__ void sum_rows(const CombineArgs *pa, int d, int N, un
     E *grp = reinterpret_cast<E *>(raw);
     const int G = pa->part_G;
     const size_t nh = (size_t)pa->part_nh;
-    const RowGroups rg = row_groups((int)blockDim.x, N, c32, sizeof(T) == 8, G, GROUP / (int)sizeof(E));
+    const RowGroups rg = row_groups((int)blockDim.x, N, V, c32, sizeof(T) == 8, G, GROUP / (int)sizeof(E));
     const int lT = rg.lT, T2 = 1 << lT, stride = rg.stride, R = rg.R, cols = N / V;
     const int t = threadIdx.x, r = row_quotient(t * V, c32), q = t - r * cols;
     if (r < R) {

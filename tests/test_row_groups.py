@@ -26,7 +26,7 @@ int main()
                 const int entries = cv::row_entries(cta == 1 ? 256 : 512, 256);
                 const int V = cv::row_vector(N, fp64);
                 for (int G = 1; G <= 2048; ++G) {
-                    const cv::RowGroups g = cv::row_groups(threads, N, cv::row_reciprocal(N), fp64, G, entries);
+                    const cv::RowGroups g = cv::row_groups(threads, N, V, cv::row_reciprocal(N), fp64, G, entries);
                     const bool ok = g.R >= 1 && g.R <= G && g.stride >= N && (g.R - 1) * g.stride + N <= entries &&
                                     g.R * (N / V) <= threads && N % V == 0 && (N << g.lT) <= threads;
                     if (!ok && bad++ < 10)
