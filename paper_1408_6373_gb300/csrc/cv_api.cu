@@ -614,6 +614,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
             std::string err;
             if (jit_sample_kernel(ctx->device, a, g->ndim, a.map.pow2 != 0, min_blocks_f32(g->ndim), &k, &err) == 0) {
                 const int grid = sample_grid(ctx, k.occ, n_grid, g, nbins, flags);
+                a.wave = 0xffffffffu / (unsigned)(ctx->sms * k.occ * kWarpsPerBlock) + 1u;
                 use_parts(grid);
                 const int tk = timer_begin(ctx);
                 cudaError_t e = launch_jit_sample(k, a, grid, ctx->stream);
@@ -628,6 +629,7 @@ static int launch_pass(cv_ctx *ctx, const cv_genz *g, int nbins, const double *e
     int occ = 0, rc = occupancy(ctx, g->ndim, nbins, flags, &occ);
     if (rc) return rc;
     const int grid = sample_grid(ctx, occ, n_grid, g, nbins, flags);
+    a.wave = 0xffffffffu / (unsigned)(ctx->sms * occ * kWarpsPerBlock) + 1u;
     use_parts(grid);
     const int tk = timer_begin(ctx);
     cudaError_t e = dispatch_sample<Real>(g->ndim, a, grid, ctx->stream);

@@ -958,14 +958,27 @@ __device__ __forceinline__ void sample_block(const SampleArgs<double> &A, const 
 
 // nsteps consecutive 32-point blocks starting at block q0, every lane's
 // words advanced past them.  The values are summed in FP32 (FP64) over
-// runs of kRun blocks, and each run's sum is added to the per-thread
-// accumulators.
+// runs of `run` blocks (even, kRun at most), and each run's sum is added to
+// the per-thread accumulators.
 //   EDGE = false: every index of the range is inside [start, end), q0 and
 //   nsteps are even; the blocks go in (even, odd) pairs, and the step out
 //   of an even block is the fixed word W_5.
 //   EDGE = true: any range (the first and last chunks of a pass), one block
 //   at a time.
 constexpr unsigned kRun = 16;
+
+// The run of a pass of nblk blocks: as many as a full wave's warps would take
+// of it each (wave = ceil(2^32 / their number)), even, kRun at most, so that
+// fewer, longer warps don't lengthen the plain sums.  (26 dimensions,
+// Gaussian, 256 bins, 5.6e5 points, whose variance is 1e-6 of its terms: its
+// error estimate is 1.3e-4 off (rms) with runs of 8 blocks, 2.8e-4 with 16.
+// In integers: a conversion of nblk to binary32 took 0.4 us of a pass.)
+__device__ __forceinline__ unsigned run_blocks(unsigned long long nblk, unsigned wave)
+{
+    if (wave == 0u || nblk > 65535ull) return kRun;
+    const unsigned k = __umulhi((unsigned)nblk - 1u, wave) + 1u;
+    return min((k + 1u) & ~1u, kRun);
+}
 
 // gp: where the integrand policy reads its parameters (the launch's
 // GenzParams, or a register copy of one integral's).
@@ -975,14 +988,14 @@ __device__ __forceinline__ void run_steps(const SampleArgs<Real> &A, const Smem<
                                           unsigned long long q0, unsigned nsteps,
                                           unsigned long long start, unsigned long long end,
                                           int lane, int hmode, Acc<Real> (&s1)[CV_MAX_COMP],
-                                          Acc<Real> (&s2)[CV_MAX_COMP], const G &gp)
+                                          Acc<Real> (&s2)[CV_MAX_COMP], const G &gp, unsigned run = kRun)
 {
     using W = typename Word<Real>::type;
     const int li = (sizeof(Real) == 4 && POW2) ? I::table(A.map) : 0;  // direction table
     const unsigned per = EDGE ? 1u : 2u;  // blocks per loop trip
     const int delay = I::delay(gp);       // (read once: the integrand-cost knob)
-    for (unsigned r0 = 0; r0 < nsteps; r0 += kRun) {
-        const unsigned r1 = min(r0 + kRun, nsteps);
+    for (unsigned r0 = 0; r0 < nsteps; r0 += run) {
+        const unsigned r1 = min(r0 + run, nsteps);
         Partial<Real> P;
         P.zero();
         for (unsigned st = r0; st < r1; st += per) {
@@ -1197,6 +1210,7 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
     // (an FP64 pass may give a warp a single block)
     if (sizeof(Real) == 4 || plen > 1) plen = (plen + 1ull) & ~1ull;
     const unsigned long long nchunk = (nblk + plen - 1) / plen;
+    const unsigned run = I::kMode == 0 && sizeof(Real) == 4 ? run_blocks(nblk, A.wave) : kRun;
     // Chunks go to warps CTA by CTA; in a pass with chunks for at most half
     // the warps, to warp 0 of every CTA, then warp 1, ..., so that every SM
     // is loaded alike.  (A full pass is 1.2% slower that way.)
@@ -1219,9 +1233,11 @@ __device__ __forceinline__ void sample_pass(const SampleArgs<Real> &A)
         }
         const bool interior = (q0 * 32ull >= start) && (q1 * 32ull <= end) && !((q0 | q1) & 1ull);
         if (interior)
-            run_steps<NDIM, Real, POW2, false, I>(A, sm, X, q0, (unsigned)(q1 - q0), start, end, lane, hmode, s1, s2, A.g);
+            run_steps<NDIM, Real, POW2, false, I>(A, sm, X, q0, (unsigned)(q1 - q0), start, end, lane, hmode, s1, s2, A.g,
+                                                  run);
         else
-            run_steps<NDIM, Real, POW2, true, I>(A, sm, X, q0, (unsigned)(q1 - q0), start, end, lane, hmode, s1, s2, A.g);
+            run_steps<NDIM, Real, POW2, true, I>(A, sm, X, q0, (unsigned)(q1 - q0), start, end, lane, hmode, s1, s2, A.g,
+                                                 run);
     }
 
     if constexpr (I::kMode == 1) return;  // points stored: nothing to reduce
@@ -1337,75 +1353,76 @@ __device__ __forceinline__ void sample_pass_owner(const SampleArgs<float> &A)
     }
 
     const int delay = I::delay(A.g);
-    Partial<float> P;
-    P.zero();
-    for (int r = 0; r < rounds; ++r) {
-        const unsigned long long group = g0 + (unsigned long long)r;
-        const unsigned long long i = group * 256ull + threadIdx.x;
-        const bool valid = i >= start && i < end;
-        float z[NDIM];
-        float J = 1.0f;
-        unsigned slot;
+    const int run = (int)run_blocks((gb - ga) * 8ull, A.wave);
+    for (int r0 = 0; r0 < rounds; r0 += run) {
+        const int r1 = min(r0 + run, rounds);
+        Partial<float> P;
+        P.zero();
+        for (int r = r0; r < r1; ++r) {
+            const unsigned long long group = g0 + (unsigned long long)r;
+            const unsigned long long i = group * 256ull + threadIdx.x;
+            const bool valid = i >= start && i < end;
+            float z[NDIM];
+            float J = 1.0f;
+            unsigned slot;
 #pragma unroll
-        for (int d = 0; d < NDIM; ++d) z[d] = map_f32<true>(X[d], d, N, A.map, sm, J, slot);
-        if (delay) J += 0.0f * delay_chain<NDIM>(z, delay * ncomp);
-        if (!valid) J = 0.0f;  // (f is finite at every point of the block)
-        const float v0 = J * genz_f32<NDIM, 0, I>(A.g, z);
-        float *buf = sq + (r & 1) * kBlock;
-        buf[threadIdx.x] = v0 * v0;
-        const float f1 = ncomp > 1 ? genz_f32<NDIM, 1, I>(A.g, z) : 0.0f;
-        const float2 v01 = make_float2(v0, J * f1);
-        P.s1[0] = add2(P.s1[0], v01);
-        P.s2[0] = fma2(v01, v01, P.s2[0]);
-        if (ncomp > 2) {
-            const float f2 = genz_f32<NDIM, 2, I>(A.g, z);
-            const float f3 = ncomp > 3 ? genz_f32<NDIM, 3, I>(A.g, z) : 0.0f;
-            const float2 v23 = make_float2(J * f2, J * f3);
-            P.s1[1] = add2(P.s1[1], v23);
-            P.s2[1] = fma2(v23, v23, P.s2[1]);
-        }
-        if ((r + 1) % (int)kRun == 0 || r + 1 == rounds) {
-#pragma unroll
-            for (int c = 0; c < CV_MAX_COMP; ++c) {
-                if (c < ncomp) {
-                    s1[c].add(P.v1(c));
-                    s2[c].add(P.v2(c));
-                }
+            for (int d = 0; d < NDIM; ++d) z[d] = map_f32<true>(X[d], d, N, A.map, sm, J, slot);
+            if (delay) J += 0.0f * delay_chain<NDIM>(z, delay * ncomp);
+            if (!valid) J = 0.0f;  // (f is finite at every point of the block)
+            const float v0 = J * genz_f32<NDIM, 0, I>(A.g, z);
+            float *buf = sq + (r & 1) * kBlock;
+            buf[threadIdx.x] = v0 * v0;
+            const float f1 = ncomp > 1 ? genz_f32<NDIM, 1, I>(A.g, z) : 0.0f;
+            const float2 v01 = make_float2(v0, J * f1);
+            P.s1[0] = add2(P.s1[0], v01);
+            P.s2[0] = fma2(v01, v01, P.s2[0]);
+            if (ncomp > 2) {
+                const float f2 = genz_f32<NDIM, 2, I>(A.g, z);
+                const float f3 = ncomp > 3 ? genz_f32<NDIM, 3, I>(A.g, z) : 0.0f;
+                const float2 v23 = make_float2(J * f2, J * f3);
+                P.s1[1] = add2(P.s1[1], v23);
+                P.s2[1] = fma2(v23, v23, P.s2[1]);
             }
-            P.zero();
-        }
-        // the step from this group's blocks to the next group's (i + 256):
-        // Gray-code bits 7 and 8 + ctz(group + 1) flip
-        const int k = 8 + min(__ffsll((long long)(group + 1ull)) - 1, CV_SOBOL_BITS - 9);
+            // the step from this group's blocks to the next group's (i + 256):
+            // Gray-code bits 7 and 8 + ctz(group + 1) flip
+            const int k = 8 + min(__ffsll((long long)(group + 1ull)) - 1, CV_SOBOL_BITS - 9);
 #pragma unroll
-        for (int d = 0; d < NDIM; ++d) X[d] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
-        __syncthreads();
-        // the group's 256 values into this warp's axes: a row starts on a
-        // multiple of its size, so the step to the next block's slot is an
-        // XOR of the address itself
-        float h[kWarpsPerBlock];
+            for (int d = 0; d < NDIM; ++d) X[d] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
+            __syncthreads();
+            // the group's 256 values into this warp's axes: a row starts on a
+            // multiple of its size, so the step to the next block's slot is an
+            // XOR of the address itself
+            float h[kWarpsPerBlock];
 #pragma unroll
-        for (int w = 0; w < kWarpsPerBlock; ++w) h[w] = buf[w * 32 + lane];
-        unsigned at[kOwn];
-#pragma unroll
-        for (int j = 0; j < kOwn; ++j) {
-            const int d = own(j);
-            at[j] = __funnelshift_r(O[j], sm.h_hi + (unsigned)d, A.map.sA + 1u);
-            O[j] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
-        }
-#pragma unroll
-        for (int w = 0; w < kWarpsPerBlock; ++w) {
-            float v[kOwn];
-#pragma unroll
-            for (int j = 0; j < kOwn; ++j)
-                if (warp + 8 * j < NDIM) v[j] = lds_f(at[j]);
+            for (int w = 0; w < kWarpsPerBlock; ++w) h[w] = buf[w * 32 + lane];
+            unsigned at[kOwn];
 #pragma unroll
             for (int j = 0; j < kOwn; ++j) {
-                if (warp + 8 * j < NDIM) sts_f(at[j], v[j] + h[w]);
-                // (out of block w of the group: bits 4 and 5 + ctz(w + 1) flip)
-                if (w < 7) at[j] ^= step[j][w & 1 ? (w == 3 ? 2 : 1) : 0];
+                const int d = own(j);
+                at[j] = __funnelshift_r(O[j], sm.h_hi + (unsigned)d, A.map.sA + 1u);
+                O[j] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
             }
-            __syncwarp();
+#pragma unroll
+            for (int w = 0; w < kWarpsPerBlock; ++w) {
+                float v[kOwn];
+#pragma unroll
+                for (int j = 0; j < kOwn; ++j)
+                    if (warp + 8 * j < NDIM) v[j] = lds_f(at[j]);
+#pragma unroll
+                for (int j = 0; j < kOwn; ++j) {
+                    if (warp + 8 * j < NDIM) sts_f(at[j], v[j] + h[w]);
+                    // (out of block w of the group: bits 4 and 5 + ctz(w + 1) flip)
+                    if (w < 7) at[j] ^= step[j][w & 1 ? (w == 3 ? 2 : 1) : 0];
+                }
+                __syncwarp();
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < CV_MAX_COMP; ++c) {
+            if (c < ncomp) {
+                s1[c].add(P.v1(c));
+                s2[c].add(P.v2(c));
+            }
         }
     }
     __syncthreads();

@@ -286,11 +286,12 @@ struct SampleArgs {
     // a reduction after a standalone pass).  Null: FP64 atomics, whose
     // order varies from run to run.
     // (16-byte aligned: the batched kernel keeps a tile in its staged copy's
-    // place of these four)
+    // place of these and the next)
     alignas(16) double *part_S;     // [part_G][2 CV_MAX_COMP]
     void *part_H;                   // [part_G][ndim][nbins]
     unsigned *part_ticket;
     int part_G;
+    unsigned wave;                  // ceil(2^32 / warps of a full wave), or 0: see run_blocks
 };
 
 // Bytes of the per-block partials of a deterministic pass.
