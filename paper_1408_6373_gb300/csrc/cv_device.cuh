@@ -1354,75 +1354,77 @@ __device__ __forceinline__ void sample_pass_owner(const SampleArgs<float> &A)
 
     const int delay = I::delay(A.g);
     const int run = (int)run_blocks((gb - ga) * 8ull, A.wave);
-    for (int r0 = 0; r0 < rounds; r0 += run) {
-        const int r1 = min(r0 + run, rounds);
-        Partial<float> P;
-        P.zero();
-        for (int r = r0; r < r1; ++r) {
-            const unsigned long long group = g0 + (unsigned long long)r;
-            const unsigned long long i = group * 256ull + threadIdx.x;
-            const bool valid = i >= start && i < end;
-            float z[NDIM];
-            float J = 1.0f;
-            unsigned slot;
+    int next = min(run, rounds);  // (the round after which the plain sums are folded)
+    Partial<float> P;
+    P.zero();
+    for (int r = 0; r < rounds; ++r) {
+        const unsigned long long group = g0 + (unsigned long long)r;
+        const unsigned long long i = group * 256ull + threadIdx.x;
+        const bool valid = i >= start && i < end;
+        float z[NDIM];
+        float J = 1.0f;
+        unsigned slot;
 #pragma unroll
-            for (int d = 0; d < NDIM; ++d) z[d] = map_f32<true>(X[d], d, N, A.map, sm, J, slot);
-            if (delay) J += 0.0f * delay_chain<NDIM>(z, delay * ncomp);
-            if (!valid) J = 0.0f;  // (f is finite at every point of the block)
-            const float v0 = J * genz_f32<NDIM, 0, I>(A.g, z);
-            float *buf = sq + (r & 1) * kBlock;
-            buf[threadIdx.x] = v0 * v0;
-            const float f1 = ncomp > 1 ? genz_f32<NDIM, 1, I>(A.g, z) : 0.0f;
-            const float2 v01 = make_float2(v0, J * f1);
-            P.s1[0] = add2(P.s1[0], v01);
-            P.s2[0] = fma2(v01, v01, P.s2[0]);
-            if (ncomp > 2) {
-                const float f2 = genz_f32<NDIM, 2, I>(A.g, z);
-                const float f3 = ncomp > 3 ? genz_f32<NDIM, 3, I>(A.g, z) : 0.0f;
-                const float2 v23 = make_float2(J * f2, J * f3);
-                P.s1[1] = add2(P.s1[1], v23);
-                P.s2[1] = fma2(v23, v23, P.s2[1]);
-            }
-            // the step from this group's blocks to the next group's (i + 256):
-            // Gray-code bits 7 and 8 + ctz(group + 1) flip
-            const int k = 8 + min(__ffsll((long long)(group + 1ull)) - 1, CV_SOBOL_BITS - 9);
+        for (int d = 0; d < NDIM; ++d) z[d] = map_f32<true>(X[d], d, N, A.map, sm, J, slot);
+        if (delay) J += 0.0f * delay_chain<NDIM>(z, delay * ncomp);
+        if (!valid) J = 0.0f;  // (f is finite at every point of the block)
+        const float v0 = J * genz_f32<NDIM, 0, I>(A.g, z);
+        float *buf = sq + (r & 1) * kBlock;
+        buf[threadIdx.x] = v0 * v0;
+        const float f1 = ncomp > 1 ? genz_f32<NDIM, 1, I>(A.g, z) : 0.0f;
+        const float2 v01 = make_float2(v0, J * f1);
+        P.s1[0] = add2(P.s1[0], v01);
+        P.s2[0] = fma2(v01, v01, P.s2[0]);
+        if (ncomp > 2) {
+            const float f2 = genz_f32<NDIM, 2, I>(A.g, z);
+            const float f3 = ncomp > 3 ? genz_f32<NDIM, 3, I>(A.g, z) : 0.0f;
+            const float2 v23 = make_float2(J * f2, J * f3);
+            P.s1[1] = add2(P.s1[1], v23);
+            P.s2[1] = fma2(v23, v23, P.s2[1]);
+        }
+        if (r + 1 == next) {
+            next = min(next + run, rounds);
 #pragma unroll
-            for (int d = 0; d < NDIM; ++d) X[d] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
-            __syncthreads();
-            // the group's 256 values into this warp's axes: a row starts on a
-            // multiple of its size, so the step to the next block's slot is an
-            // XOR of the address itself
-            float h[kWarpsPerBlock];
-#pragma unroll
-            for (int w = 0; w < kWarpsPerBlock; ++w) h[w] = buf[w * 32 + lane];
-            unsigned at[kOwn];
-#pragma unroll
-            for (int j = 0; j < kOwn; ++j) {
-                const int d = own(j);
-                at[j] = __funnelshift_r(O[j], sm.h_hi + (unsigned)d, A.map.sA + 1u);
-                O[j] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
-            }
-#pragma unroll
-            for (int w = 0; w < kWarpsPerBlock; ++w) {
-                float v[kOwn];
-#pragma unroll
-                for (int j = 0; j < kOwn; ++j)
-                    if (warp + 8 * j < NDIM) v[j] = lds_f(at[j]);
-#pragma unroll
-                for (int j = 0; j < kOwn; ++j) {
-                    if (warp + 8 * j < NDIM) sts_f(at[j], v[j] + h[w]);
-                    // (out of block w of the group: bits 4 and 5 + ctz(w + 1) flip)
-                    if (w < 7) at[j] ^= step[j][w & 1 ? (w == 3 ? 2 : 1) : 0];
+            for (int c = 0; c < CV_MAX_COMP; ++c) {
+                if (c < ncomp) {
+                    s1[c].add(P.v1(c));
+                    s2[c].add(P.v2(c));
                 }
-                __syncwarp();
             }
+            P.zero();
+        }
+        // the step from this group's blocks to the next group's (i + 256):
+        // Gray-code bits 7 and 8 + ctz(group + 1) flip
+        const int k = 8 + min(__ffsll((long long)(group + 1ull)) - 1, CV_SOBOL_BITS - 9);
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d) X[d] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
+        __syncthreads();
+        // the group's 256 values into this warp's axes: a row starts on a
+        // multiple of its size, so the step to the next block's slot is an
+        // XOR of the address itself
+        float h[kWarpsPerBlock];
+#pragma unroll
+        for (int w = 0; w < kWarpsPerBlock; ++w) h[w] = buf[w * 32 + lane];
+        unsigned at[kOwn];
+#pragma unroll
+        for (int j = 0; j < kOwn; ++j) {
+            const int d = own(j);
+            at[j] = __funnelshift_r(O[j], sm.h_hi + (unsigned)d, A.map.sA + 1u);
+            O[j] ^= Dir<unsigned>::w(li, d, 7) ^ Dir<unsigned>::w(li, d, k);
         }
 #pragma unroll
-        for (int c = 0; c < CV_MAX_COMP; ++c) {
-            if (c < ncomp) {
-                s1[c].add(P.v1(c));
-                s2[c].add(P.v2(c));
+        for (int w = 0; w < kWarpsPerBlock; ++w) {
+            float v[kOwn];
+#pragma unroll
+            for (int j = 0; j < kOwn; ++j)
+                if (warp + 8 * j < NDIM) v[j] = lds_f(at[j]);
+#pragma unroll
+            for (int j = 0; j < kOwn; ++j) {
+                if (warp + 8 * j < NDIM) sts_f(at[j], v[j] + h[w]);
+                // (out of block w of the group: bits 4 and 5 + ctz(w + 1) flip)
+                if (w < 7) at[j] ^= step[j][w & 1 ? (w == 3 ? 2 : 1) : 0];
             }
+            __syncwarp();
         }
     }
     __syncthreads();
